@@ -134,9 +134,11 @@ typedef struct {
  * call only).  Allocates the device state.  *out receives the context.
  * Euler equations with GRPrec of degree 2 or 4, the TT solver and no source:
  * the flux phase solves the Riemann problems that are not equal data in a
- * second kernel, from a list of n_if / 4 + 1024 interfaces (n_if = the total
- * interface count) held by the context, (6 (M + 1) + 1) x 8 bytes each;
- * interfaces beyond it are solved in the first kernel.
+ * second kernel, from a list held by the context (4 bytes for every
+ * interface).  At degree 2, with gamma in [1.2, 1.9] and the FLAT form, the
+ * first kernel computes in 64-bit fixed point, each interface in its own powers
+ * of two (rounding errors below those of FP64); interfaces that leave that
+ * format's range are solved in FP64 by the second kernel.
  * Errors: GRP_E_INVALID_ARG for any field outside its range, GRP_E_CUDA.
  */
 int grp_create(grp_ctx **out, const grp_problem *p);

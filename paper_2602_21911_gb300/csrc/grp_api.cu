@@ -37,8 +37,7 @@ struct grp_ctx {
   DomStep* ds = nullptr;         // per-domain time step of the current step
   double* det_ed = nullptr;      // DET: evolved edge values of every cell
   double* srcv = nullptr;        // numerical source of every cell (source terms only)
-  double* hard_tr = nullptr;     // flux kernel's deferred interfaces: traces, index, counters
-  long long* hard_idx = nullptr;
+  int* hard_idx = nullptr;       // flux kernel's deferred interfaces, and its counters
   unsigned* hard_count = nullptr;
   long long hard_cap = 0;
   // admissibility flags of the interface data, one buffer per state buffer;
@@ -137,7 +136,7 @@ void free_all(grp_ctx* c)
                   c->status, c->smax_bits, c->bad, c->inad, c->fail, c->any_bad, c->tlist0, c->tlist1,
                   c->ilist, c->lcount, c->stats,
                   c->scratch_norm, c->mlp, c->mlp_norm, c->grp, c->tiles, c->tile_zeros, c->tile_flag,
-                  c->hard_tr, c->hard_idx, c->hard_count, c->gadm[0], c->gadm[1]};
+                  c->hard_idx, c->hard_count, c->gadm[0], c->gadm[1]};
   for (void* q : ptrs)
     if (q) cudaFree(q);
 }
@@ -194,10 +193,13 @@ StepArgs make_args(const grp_ctx* c, double t_end)
   a.harvest_cap = c->harvest_cap;
   a.harvest_log2_stride = c->harvest_log2_stride;
   a.srcv = c->srcv;
-  a.hard_tr = c->hard_tr;
   a.hard_idx = c->hard_idx;
   a.hard_count = c->hard_count;
   a.hard_cap = (int)c->hard_cap;
+  if (fixed::gamma_ok(a.ph.gamma)) {
+    a.fx_gm1 = fixed::to_format(a.ph.gm1);
+    a.fx_hgam = fixed::to_format(0.5 * a.ph.gamma);
+  }
   a.ph.src = c->p.source;
   a.ph.src_k = c->p.source_coef;
   return a;
@@ -437,14 +439,19 @@ int enqueue_step(grp_ctx* c, double t_end)
 {
   c->smax_ready = false;
   StepArgs a = make_args(c, t_end);
+  cudaStream_t s = c->stream;
   // the flat flux kernel at degrees 2 and 4 keeps the interface data's
-  // admissibility flags; the first step after new data tests the data
+  // admissibility flags; after a step of another form they are formed anew
   const bool flags = c->gadm[0] && flux_defers(a);
   if (flags) {
-    a.adm_in = c->adm_valid ? c->gadm[c->cur] : nullptr;
+    if (!c->adm_valid) {
+      k_adm<<<blocks(c->nif, 256), 256, 0, s>>>(c->p.gamma, c->nif, a.ifc, c->gadm[c->cur]);
+      c->launches++;
+    }
+    a.adm_in = c->gadm[c->cur];
     a.adm_out = c->gadm[c->cur ^ 1];
+    a.fixed = flux_fixed(a) ? 1 : 0;
   }
-  cudaStream_t s = c->stream;
   const bool euler = c->p.system == GRP_EULER_IDEAL;
   if (euler) {
     k_smax<<<blocks(c->ncell, 256), 256, 0, s>>>(a);
@@ -603,8 +610,8 @@ int grp_create(grp_ctx** out, const grp_problem* p)
   if (p->source != GRP_SOURCE_NONE) AL(srcv, (long long)C * c->ncell)
   if (p->system == GRP_EULER_IDEAL && p->recon == GRP_RECON_GRPREC && p->solver != GRP_SOLVER_DET &&
       p->source == GRP_SOURCE_NONE && (p->M == 2 || p->M == 4)) {
-    c->hard_cap = hard_list_cap(c->nif);
-    AL(hard_tr, (long long)hard_doubles_per_slot(p->M) * c->hard_cap) AL(hard_idx, c->hard_cap) AL(hard_count, 3)
+    c->hard_cap = c->nif;
+    AL(hard_idx, c->hard_cap) AL(hard_count, 3)
     AL(gadm[0], c->nif) AL(gadm[1], c->nif)
     if ((e = cudaMemset(c->hard_count, 0, 3 * sizeof(unsigned))) != cudaSuccess) {
       free_all(c); delete c; return cuda_fail(e, "cudaMemset hard_count");
@@ -660,7 +667,8 @@ int grp_set_initial(grp_ctx* c, const double* averages, const double* lim_minus,
     CK(cudaMemcpyAsync(lm, lim_minus, sizeof(double) * c->C * c->nif, k, s));
     CK(cudaMemcpyAsync(lp, lim_plus, sizeof(double) * c->C * c->nif, k, s));
     const Phys ph = make_phys(c->p.lambda, c->p.gamma, c->p.newton_rtol, c->p.newton_max_iter, 0);
-    k_init_iface<<<blocks(c->nif, 128), 128, 0, s>>>(c->p.system, ph, c->nif, lm, lp, c->ifc[0]);
+    k_init_iface<<<blocks(c->nif, 128), 128, 0, s>>>(c->p.system, ph, c->nif, lm, lp, c->ifc[0], c->gadm[0]);
+    c->adm_valid = c->gadm[0] != nullptr;
     c->launches++;
     CK(cudaGetLastError());
   }

@@ -7,6 +7,17 @@
 #include "grp_launch.h"
 
 namespace grp {
+// the first pass in fixed point, where the caller chose it (flux_fixed)
+template <int MM, bool NLV>
+inline bool launch_flux_fixed(const StepArgs& a, cudaStream_t s)
+{
+  if constexpr (MM == 2 && !NLV) {
+    if (a.fixed) k_flux_fixed<MM><<<(unsigned)((a.nif + 127) / 128), 128, 0, s>>>(a);
+    return a.fixed != 0;
+  }
+  return false;
+}
+
 // the second pass of the flux kernel, where the first defers interfaces
 template <int MM, bool NLV>
 inline void launch_flux_hard(const StepArgs& a, cudaStream_t s)
@@ -36,7 +47,8 @@ inline void launch_flux_hard(const StepArgs& a, cudaStream_t s)
   cudaError_t launch_flux_euler_##SUFFIX(const StepArgs& a, cudaStream_t s)                                  \
   {                                                                                                          \
     const unsigned g = (unsigned)((flux_threads(a.nif) + GRP_FLUX_TPB - 1) / GRP_FLUX_TPB);                  \
-    if (a.ph.gamma == 1.4) k_flux<SYS_EULER, MM, true, NLV><<<g, GRP_FLUX_TPB, 0, s>>>(a);                   \
+    if (launch_flux_fixed<MM, NLV>(a, s)) {}                                                                 \
+    else if (a.ph.gamma == 1.4) k_flux<SYS_EULER, MM, true, NLV><<<g, GRP_FLUX_TPB, 0, s>>>(a);              \
     else k_flux<SYS_EULER, MM, false, NLV><<<g, GRP_FLUX_TPB, 0, s>>>(a);                                    \
     launch_flux_hard<MM, NLV>(a, s);                                                                         \
     return cudaGetLastError();                                                                               \

@@ -1,0 +1,66 @@
+"""The fixed-point first pass of the flux phase (degree 2 of the Euler
+equations, flat form) against the oracle: both flow directions, resting and
+supersonic gas, states of very large and very small units, the ratios of
+specific heats at and beyond the ends of its range, domains around the block
+size, and data that leave the format and go to the second pass."""
+import numpy as np
+import pytest
+
+from paper_2602_21911_gb300 import inputs as I
+
+from parity import DISC_TOL, SMOOTH_TOL, check_parity
+
+pytestmark = pytest.mark.gpu
+
+
+def _wave(N, u, gamma=1.4, amp=0.2, mass=1.0, speed=1.0, bc=I.PERIODIC):
+    """Density wave of velocity u at p = 1, in units (mass, speed)."""
+    prob, avg, lim, _ = I.euler_wave(N, 2, amp=amp, gamma=gamma, bc=bc)
+    unit = np.array([[1.0], [speed], [speed * speed]]) * mass
+
+    def state(r):
+        return np.stack([r, r * u, np.full_like(r, 1.0 / (gamma - 1.0)) + 0.5 * r * u * u]) * unit
+    a, g = state(avg[0]), state(lim[0])
+    return prob, a, g, g.copy()
+
+
+@pytest.mark.parametrize("N", [1, 2, 3, 31, 127, 128, 129])
+@pytest.mark.parametrize("bc", [I.PERIODIC, I.TRANSMISSIVE])
+def test_domain_sizes(N, bc):
+    check_parity(*_wave(N, -0.7, bc=bc), 20, SMOOTH_TOL)
+
+
+@pytest.mark.parametrize("u", [0.3, -0.3, 2.5, -2.5, 400.0])
+def test_flow_directions(u):
+    check_parity(*_wave(64, u), 40, SMOOTH_TOL)
+
+
+@pytest.mark.parametrize("E", [2.5, 1.7320508075688772, 0.1])
+def test_a_resting_density_wave_stays_at_rest_exactly(E):
+    """Equal pressures give equal fluxes whatever the densities, so no momentum
+    forms and no average moves (not compared with the oracle, whose own
+    rounding leaves 1e-15 of momentum here)."""
+    from paper_2602_21911_gb300 import grprec
+    prob, a, g, _ = _wave(64, 0.0, amp=0.9)
+    a[2], g[2] = E, E
+    s = grprec.Solver(prob)
+    s.set_initial(a, g)
+    s.step(40)
+    a1, g1, t = s.get_state()
+    assert np.array_equal(a1, a) and np.array_equal(g1, g) and t[0] > 0
+
+
+@pytest.mark.parametrize("gamma", [1.1, 1.2, 1.3, 5.0 / 3.0, 1.9, 2.0])
+def test_ratios_of_specific_heats(gamma):
+    check_parity(*_wave(64, 0.5, gamma=gamma), 40, SMOOTH_TOL)
+
+
+@pytest.mark.parametrize("mass,speed", [(1e90, 1e20), (1e-90, 1e-20), (1e30, 1e-40), (2.0 ** -37, 2.0 ** 41)])
+def test_units(mass, speed):
+    check_parity(*_wave(65, -0.4, mass=mass, speed=speed), 20, SMOOTH_TOL)
+
+
+@pytest.mark.parametrize("ratio", [2.0, 10.0, 1000.0])
+def test_jumps_leave_the_format(ratio):
+    for WL, WR in (((1.0, 0.5, 1.0), (ratio, 0.5, 1.0)), ((1.0, -0.5, ratio), (1.0, 0.5, 1.0))):
+        check_parity(*I.riemann_problem(101, WL, WR, M=2), 30, DISC_TOL)
