@@ -34,6 +34,7 @@ struct grp_ctx {
   double* ifc[2] = {nullptr, nullptr};
   double* flux = nullptr;
   double* pold = nullptr;        // pressure of the current averages (S_max pass)
+  unsigned* slow32 = nullptr;    // per-domain FP32 lower bound of S_max (flat form)
   DomStep* ds = nullptr;         // per-domain time step of the current step
   double* det_ed = nullptr;      // DET: evolved edge values of every cell
   double* srcv = nullptr;        // numerical source of every cell (source terms only)
@@ -132,7 +133,7 @@ void free_all(grp_ctx* c)
   c->ev_free.clear();
   c->ev_pending.clear();
   void* ptrs[] = {c->cell_off, c->if_off, c->cell_dom, c->if_dom, c->dx, c->bc, c->avg[0], c->avg[1],
-                  c->ifc[0], c->ifc[1], c->flux, c->pold, c->ds, c->det_ed, c->srcv, c->low, c->troubled, c->t, c->dt_prev, c->nstep,
+                  c->ifc[0], c->ifc[1], c->flux, c->pold, c->slow32, c->ds, c->det_ed, c->srcv, c->low, c->troubled, c->t, c->dt_prev, c->nstep,
                   c->status, c->smax_bits, c->bad, c->inad, c->fail, c->any_bad, c->tlist0, c->tlist1,
                   c->ilist, c->lcount, c->stats,
                   c->scratch_norm, c->mlp, c->mlp_norm, c->grp, c->tiles, c->tile_zeros, c->tile_flag,
@@ -167,6 +168,10 @@ StepArgs make_args(const grp_ctx* c, double t_end)
   a.ifc_new = c->ifc[c->cur ^ 1];
   a.flux = c->flux;
   a.pold = c->pold;
+  a.rp32 = (float2*)c->pold;     // one or the other: the flat form keeps FP32 pairs in the same array
+  a.sup32 = (float*)c->tlist1;   // free until the step's repair
+  a.slow32 = c->slow32;
+  a.gm1f = (float)a.ph.gm1; a.gammaf = (float)a.ph.gamma; a.h_gm1f = (float)a.ph.h_gm1;
   a.ds = c->ds;
   a.low = c->low;
   a.troubled = c->troubled;
@@ -454,8 +459,14 @@ int enqueue_step(grp_ctx* c, double t_end)
   }
   const bool euler = c->p.system == GRP_EULER_IDEAL;
   if (euler) {
-    k_smax<<<blocks(c->ncell, 256), 256, 0, s>>>(a);
-    c->launches++;
+    if (c->ncell <= SPEED_SMALL) {
+      k_speed<<<blocks(c->ncell, 256), 256, 0, s>>>(a);
+      c->launches++;
+    } else {
+      k_speed32<<<speed_blocks(c->ncell), 256, 0, s>>>(a);
+      k_speed64<<<blocks(c->ncell, 256), 256, 0, s>>>(a);
+      c->launches += 2;
+    }
   }
   k_dt<<<blocks(c->D, 128), 128, 0, s>>>(a);
   c->launches++;
@@ -603,7 +614,7 @@ int grp_create(grp_ctx** out, const grp_problem* p)
   }
   AL(cell_off, D + 1) AL(if_off, D + 1) AL(cell_dom, c->ncell) AL(if_dom, c->nif) AL(dx, D) AL(bc, D)
   AL(avg[0], C * c->ncell) AL(avg[1], C * c->ncell) AL(ifc[0], C * c->nif) AL(ifc[1], C * c->nif)
-  AL(flux, C * c->nif) AL(pold, c->ncell) AL(ds, D) AL(low, c->nif) AL(troubled, c->ncell) AL(t, D) AL(dt_prev, D) AL(nstep, D)
+  AL(flux, C * c->nif) AL(pold, c->ncell) AL(slow32, D) AL(ds, D) AL(low, c->nif) AL(troubled, c->ncell) AL(t, D) AL(dt_prev, D) AL(nstep, D)
   AL(status, D) AL(smax_bits, D) AL(bad, (MAX_REPAIR + 1) * D) AL(inad, D) AL(fail, D)
   AL(any_bad, MAX_REPAIR + 1) AL(stats, (long long)NSTATS * D) AL(scratch_norm, 3 * D)
   AL(tlist0, c->ncell) AL(tlist1, c->ncell) AL(ilist, c->nif) AL(lcount, 2 * (MAX_REPAIR + 1))
@@ -678,6 +689,7 @@ int grp_set_initial(grp_ctx* c, const double* averages, const double* lim_minus,
   CK(cudaMemsetAsync(c->nstep, 0, sizeof(int) * D, s));
   CK(cudaMemsetAsync(c->status, 0, sizeof(int) * D, s));
   CK(cudaMemsetAsync(c->smax_bits, 0, sizeof(unsigned long long) * D, s));
+  CK(cudaMemsetAsync(c->slow32, 0, sizeof(unsigned) * D, s));
   CK(cudaMemsetAsync(c->stats, 0, sizeof(unsigned long long) * NSTATS * D, s));
   CK(cudaMemsetAsync(c->low, 0, c->nif, s));
   CK(cudaMemsetAsync(c->troubled, 0, c->ncell, s));

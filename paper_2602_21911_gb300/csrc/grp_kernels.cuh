@@ -1,7 +1,8 @@
 // Kernels of one FV+GRPrec time step over a flat batch of 1D domains.
 //
 // One step is a short fixed sequence of launches on the context's stream:
-//   k_smax         per cell   S_max of every domain (warp max + atomicMax)
+//   k_speed32      per cell   FP32 bounds of |u| + c, density and pressure in FP32
+//   k_speed64      per cell   S_max of every domain from the cells that can hold it
 //   k_flux<M>      per iface  GRPrec traces -> GRP -> flux, new interface data
 //   k_update       per cell   candidate averages, detection flags, list of troubled cells
 //   k_repair_list  per listed troubled cell: first-order fluxes on its interfaces
@@ -50,7 +51,12 @@ struct StepArgs {
   double* ifc_new;                   // next interface data    [C][nif]
   double* flux;                      // scratch [C][nif]
   double* srcv = nullptr;            // [C][ncell] numerical source of every cell this step, or null (S = 0)
-  double* pold;                      // [ncell] pressure of the current averages, written with S_max
+  double* pold;                      // [ncell] pressure of the current averages, written with S_max (block-local forms)
+  float2* rp32 = nullptr;            // [ncell] flat form: density and pressure of the current averages in FP32, the
+                                     //   pressure NaN where FP32 cannot resolve it (k_speed32)
+  float gm1f, gammaf, h_gm1f;        // gamma - 1, gamma, (gamma - 1) / 2 in FP32
+  float* sup32 = nullptr;            // [ncell] flat form: an upper bound of |u| + c of every cell
+  unsigned* slow32 = nullptr;        // [D] flat form: the largest lower bound of |u| + c, as float bits
   DomStep* ds;                       // [D] this step's time step of every domain (k_dt or in-block)
   unsigned char* low;                // [nif] 0 high order; 1 first order (flux kernel); 2+r repaired in round r
   unsigned char* troubled;           // [ncell] 0 ok; 1 outside the relaxed DMP; 2 inadmissible
@@ -262,6 +268,130 @@ static __global__ void k_smax(StepArgs a)
   if (valid && gi == a.cell_off[a.cell_dom[gi]]) reset_domain_words(a, a.cell_dom[gi]);
   if (a.sys != SYS_EULER) return;                  // uniform
   smax_cell(a, gi, valid);
+}
+
+// -------------------------------------------------- S_max of the flat form
+// |u| + c and the pressure of a cell average in FP64 (an ulp or two from the
+// correctly rounded divisions and root); c = 0 without a sound speed, the
+// bits of 0 when the sum is not a number.
+__device__ __forceinline__ double cell_pressure(const StepArgs& a, double r, double m, double E, double& u, double& ir)
+{
+  ir = rcp64(r);
+  u = m * ir;
+  return a.ph.gm1 * (E - 0.5 * m * u);
+}
+
+// x in FP32, truncated (off the FP64 pipe); infinite beyond the FP32 range.
+__device__ __forceinline__ float trunc32(double x)
+{
+  const int h = __double2hiint(x), ah = h & 0x7fffffff;
+  const unsigned t = ((unsigned)(ah - (896 << 20)) << 3) | ((unsigned)__double2loint(x) >> 29);
+  const unsigned v = ah < (897 << 20) ? 0u : ah >= (1150 << 20) ? 0x7f800000u : t;
+  return __uint_as_float(v | ((unsigned)h & 0x80000000u));
+}
+
+// FP32 pass: density and pressure of every cell for the update's maximum
+// principle, and bounds of |u| + c.  FP32 decides which cells can hold the
+// domain's maximum, the second pass evaluates those in FP64, so S_max is the
+// FP64 maximum of all cells, bit for bit.  On this GPU an FP64 instruction
+// holds its pipe 16 cycles; the pass in FP64 took 17 of them per cell.
+//   Errors: with values truncated to FP32 the pressure is off by less than
+//   2^-20 (g - 1) E.  Where p > 2^-9 (g - 1) E it is therefore known to 2^-11,
+//   and |u| + c to less than that: bounds at 1 -+ 2^-10; where p > 2^-4 (g - 1) E
+//   (Mach numbers below about 5) to 2^-16: bounds at 1 -+ 2^-15.  Elsewhere (Mach
+//   numbers beyond about 30) p < 2^-8 (g - 1) E: |u| below, |u| plus that sound
+//   speed above.  What FP32 cannot hold gets the bounds 0 and infinity.
+// Several cells per thread (a block apart) keep their loads in flight together.
+constexpr int SPEED_CELLS = 4;
+inline unsigned speed_blocks(long long ncell) { return (unsigned)((ncell + 256 * SPEED_CELLS - 1) / (256 * SPEED_CELLS)); }
+
+static __global__ void __launch_bounds__(256) k_speed32(StepArgs a)
+{
+  if (blockIdx.x == 0 && threadIdx.x <= MAX_REPAIR) a.any_bad[threadIdx.x] = 0;
+  if (blockIdx.x == 0 && threadIdx.x < 2 * (MAX_REPAIR + 1)) a.lcount[threadIdx.x] = 0;
+  const long long g0 = (long long)blockIdx.x * (256 * SPEED_CELLS) + threadIdx.x;
+  double r[SPEED_CELLS], m[SPEED_CELLS], E[SPEED_CELLS];
+  int d[SPEED_CELLS];
+#pragma unroll
+  for (int k = 0; k < SPEED_CELLS; ++k) {
+    const long long gi = g0 + 256 * k;
+    d[k] = -1;
+    if (gi < a.ncell) { d[k] = a.cell_dom[gi]; r[k] = a.avg[gi]; m[k] = a.avg[a.ncell + gi]; E[k] = a.avg[2 * a.ncell + gi]; }
+  }
+#pragma unroll
+  for (int k = 0; k < SPEED_CELLS; ++k) {
+    const long long gi = g0 + 256 * k;
+    unsigned low = 0u;
+    if (d[k] >= 0) {
+      const float rf = trunc32(r[k]), mf = trunc32(m[k]), Ef = trunc32(E[k]);
+      const float ir = __fdividef(1.0f, rf), u = mf * ir, cap = a.gm1f * Ef;
+      const float p = a.gm1f * fmaf(-0.5f * mf, u, Ef);
+      const bool known = p > cap * 0x1p-9f;
+      const float au = fabsf(u), s = au + __fsqrt_rn(a.gammaf * (known ? p : cap * 0x1p-8f) * ir);
+      const float tol = p > cap * 0x1p-4f ? 0x1p-15f : 0x1p-10f;
+      float sl = (known ? s : au) * (1.0f - tol), su = s * (1.0f + tol);
+      if (!(rf > 1e-30f && cap > 1e-30f && su < 1e30f)) { sl = 0.0f; su = INFINITY; }
+      a.rp32[gi] = make_float2(rf, known && su < 1e30f ? p : NAN);
+      a.sup32[gi] = su;
+      low = __float_as_uint(sl);
+    }
+    const unsigned grp = __match_any_sync(0xffffffffu, d[k]);
+    const unsigned mx = __reduce_max_sync(grp, low);
+    if (d[k] >= 0 && lane_id() == __ffs(grp) - 1) atomicMax(a.slow32 + d[k], mx);
+  }
+}
+
+// Both in one FP64 launch, for grids that leave the GPU mostly idle (the two
+// passes' latencies add up there: 7 us on a domain of 200 cells).
+constexpr long long SPEED_SMALL = 1 << 17;
+static __global__ void __launch_bounds__(256) k_speed(StepArgs a)
+{
+  if (blockIdx.x == 0 && threadIdx.x <= MAX_REPAIR) a.any_bad[threadIdx.x] = 0;
+  if (blockIdx.x == 0 && threadIdx.x < 2 * (MAX_REPAIR + 1)) a.lcount[threadIdx.x] = 0;
+  const long long gi = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  int d = -1;
+  unsigned hi = 0u, lo = 0u;
+  if (gi < a.ncell) {
+    d = a.cell_dom[gi];
+    const double r = a.avg[gi], m = a.avg[a.ncell + gi], E = a.avg[2 * a.ncell + gi];
+    double u, ir;
+    const double p = cell_pressure(a, r, m, E, u, ir);
+    const double c2 = a.ph.gamma * p * ir;
+    const double sp = fabs(u) + (positive(c2) ? c2 * rsqrt(c2) : 0.0);
+    const long long sb = __double_as_longlong(sp);
+    if (sb >= 0ll && sb <= 0x7ff0000000000000ll) { hi = (unsigned)(sb >> 32); lo = (unsigned)sb; }
+    const float rf = trunc32(r), pf = trunc32(p), cap = a.gm1f * trunc32(E);
+    a.rp32[gi] = make_float2(rf, rf > 1e-30f && cap > 1e-30f && cap < 1e30f && pf > cap * 0x1p-9f ? pf : NAN);
+  }
+  // the largest 64-bit pattern of the warp's cells of one domain, in two words
+  const unsigned grp = __match_any_sync(0xffffffffu, d);
+  const unsigned mh = __reduce_max_sync(grp, hi);
+  const unsigned ml = __reduce_max_sync(grp, hi == mh ? lo : 0u);
+  if (d >= 0 && lane_id() == __ffs(grp) - 1)
+    atomicMax(a.smax_bits + d, ((unsigned long long)mh << 32) | ml);
+}
+
+// FP64 pass over the cells that can hold the maximum.  Runs of identical
+// states (undisturbed gas) are evaluated at their first cell.
+static __global__ void __launch_bounds__(256) k_speed64(StepArgs a)
+{
+  const long long gi = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (gi >= a.ncell) return;
+  const int d = a.cell_dom[gi];
+  if (a.sup32[gi] < __uint_as_float(a.slow32[d])) return;
+  const double r = a.avg[gi], m = a.avg[a.ncell + gi], E = a.avg[2 * a.ncell + gi];
+  if (gi > a.cell_off[d]) {
+    const long long dr = __double_as_longlong(r) ^ __double_as_longlong(a.avg[gi - 1]);
+    const long long dm = __double_as_longlong(m) ^ __double_as_longlong(a.avg[a.ncell + gi - 1]);
+    const long long dE = __double_as_longlong(E) ^ __double_as_longlong(a.avg[2 * a.ncell + gi - 1]);
+    if ((dr | dm | dE) == 0) return;
+  }
+  double u, ir;
+  const double p = cell_pressure(a, r, m, E, u, ir);
+  const double c2 = a.ph.gamma * p * ir;
+  const double sp = fabs(u) + (positive(c2) ? c2 * rsqrt(c2) : 0.0);
+  const long long sb = __double_as_longlong(sp);
+  if (sb >= 0ll && sb <= 0x7ff0000000000000ll) atomicMax(a.smax_bits + d, (unsigned long long)sb);
 }
 
 // ------------------------------------------------------------------ traces
@@ -922,6 +1052,31 @@ __global__ void __launch_bounds__(GRP_HARD_TPB, GRP_HARD_MIN_BLOCKS) k_flux_hard
 }
 
 // ------------------------------------------------------------------ update
+// What FP32 shows of the candidate Q of a cell: 0 admissible and inside the
+// relaxed maximum principle (see update_one), 1 admissible and outside it, -1 not
+// decided.  x, y, z: density and pressure of the old averages of cells i - 1, i,
+// i + 1.  With Q truncated to 2^-23 the term 2 E rho - m^2 is off by less than
+// 2^-20 of 2 E rho, the old density by 2^-23 and the old pressure by 2^-11; the
+// margins (2^-18 of the density bound, 2^-9 of the pressure bound) cover them.
+// Comparisons are written to leave NaN undecided.
+__device__ __forceinline__ int dmp32(const StepArgs& a, float2 x, float2 y, float2 z, const double Q[3])
+{
+  const float rlo = fminf(fminf(x.x, y.x), z.x), rhi = fmaxf(fmaxf(x.x, y.x), z.x);
+  const float plo = fminf(fminf(x.y, y.y), z.y), phi = fmaxf(fmaxf(x.y, y.y), z.y);
+  const float r = trunc32(Q[0]), m = trunc32(Q[1]), E2 = 2.0f * trunc32(Q[2]);
+  const float A = E2 * r, a2 = fmaf(E2, r, -(m * m)), ea = A * 0x1p-20f, pb = phi * r;
+  const float rel = (float)DMP_REL, rp = a.h_gm1f * a2, erp = a.h_gm1f * ea;
+  if (!(x.y + y.y + z.y < INFINITY && r > 0.0f && a2 > ea && A > 1e-30f && A < 1e30f && pb > 1e-30f && pb < 1e30f))
+    return -1;
+  // distances inside the four ends of the band, less and plus their margins
+  const float sr = 0x1p-18f * rhi, sp = fmaf(0x1p-9f, pb, erp);
+  const float q0 = fmaf(rel, rhi, r - rlo), q1 = fmaf(rel, rhi, rhi - r);
+  const float q2 = fmaf(rel, pb, rp - plo * r), q3 = fmaf(rel, pb, pb - rp);
+  const float qr = fminf(q0, q1), qp = fminf(q2, q3);
+  if (qr >= sr && qp >= sp) return 0;
+  return qr < -sr || qp < -sp ? 1 : -1;
+}
+
 // Candidate average of cell gi from the flux array, with the a-posteriori
 // detection: inadmissible, or outside the relaxed discrete maximum principle
 // on density and pressure against the old averages of cells i-1, i, i+1.
@@ -929,7 +1084,11 @@ __global__ void __launch_bounds__(GRP_HARD_TPB, GRP_HARD_MIN_BLOCKS) k_flux_hard
 // `pass`, which recomputes only the cells next to an interface repaired in
 // that round (every other candidate depends on unchanged fluxes).
 // Returns bit 0: troubled, bit 1: inadmissible.
-template <int SYS>
+// P32 (flat form): the old states' density and pressure are there in FP32
+// (k_speed32).  The band is 1 % wide, so FP32 with its error bounds clears
+// nearly every cell; the rest takes the FP64 test, with the old pressures formed
+// there.  The outcome is the FP64 test's in every case.
+template <int SYS, bool P32 = false>
 __device__ __forceinline__ int update_one(const StepArgs& a, long long gi, int d, int pass)
 {
   constexpr int C = SYS == SYS_EULER ? 3 : 1;
@@ -961,6 +1120,16 @@ __device__ __forceinline__ int update_one(const StepArgs& a, long long gi, int d
     a.avg_new[c * a.ncell + gi] = Q[c];
   }
   if (SYS != SYS_EULER) return 0;
+  if (P32 && pass < 0) {
+    int im, ip;
+    nbr(i, N, a.bc[d], im, ip);
+    const int f = dmp32(a, a.rp32[c0 + im], a.rp32[gi], a.rp32[c0 + ip], Q);
+    if (f >= 0) {
+      a.troubled[gi] = (unsigned char)f;
+      if (f) a.bad[d] = 1;
+      return f;
+    }
+  }
   // admissible: rho > 0 and 2 E rho - m^2 = 2 rho p / (g - 1) > 0 (the
   // latter also gives the candidate's rho p below)
   const double a2 = fma(Q[2] + Q[2], Q[0], -(Q[1] * Q[1]));
@@ -979,7 +1148,10 @@ __device__ __forceinline__ int update_one(const StepArgs& a, long long gi, int d
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       const long long q = c0 + nb[k];
-      const long long r = __double_as_longlong(a.avg[q]), pr = __double_as_longlong(a.pold[q]);
+      double pk, uk, ik;
+      if (P32) pk = cell_pressure(a, a.avg[q], a.avg[a.ncell + q], a.avg[2 * a.ncell + q], uk, ik);
+      else pk = a.pold[q];
+      const long long r = __double_as_longlong(a.avg[q]), pr = __double_as_longlong(pk);
       lo0 = k == 0 ? r : min(lo0, r); hi0 = k == 0 ? r : max(hi0, r);
       lo1 = k == 0 ? pr : min(lo1, pr); hi1 = k == 0 ? pr : max(hi1, pr);
     }
@@ -1006,13 +1178,13 @@ __device__ __forceinline__ int update_one(const StepArgs& a, long long gi, int d
 }
 
 template <int SYS>
-__global__ void k_update(StepArgs a, int pass)
+__global__ void __launch_bounds__(256, 8) k_update(StepArgs a, int pass)
 {
   const long long gi = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (pass >= 0 && a.any_bad[pass] == 0) return;
   if (gi >= a.ncell) return;
   const int d = a.cell_dom[gi];
-  const bool bad = update_one<SYS>(a, gi, d, pass) & 1;
+  const bool bad = update_one<SYS, SYS == SYS_EULER>(a, gi, d, pass) & 1;
   if (bad) a.any_bad[pass + 1] = 1;
   if (pass < 0 && a.lcount) {
     // warp-aggregated append of the troubled cells to the first work list
@@ -1129,7 +1301,7 @@ __global__ void __launch_bounds__(LIST_THREADS) k_update_list(StepArgs a, int pa
     if (cl >= 0 && a.low[i0 + cl] != mark) cells[nc++] = cl;
     for (int q = 0; q < nc; ++q) {
       const long long gi = c0 + cells[q];
-      if (update_one<SYS>(a, gi, d, pass) & 1) {
+      if (update_one<SYS, SYS == SYS_EULER>(a, gi, d, pass) & 1) {
         a.any_bad[pass + 1] = 1;
         if (pass + 1 <= MAX_REPAIR) a.tlist[(pass + 1) & 1][atomicAdd(a.lcount + pass + 1, 1)] = (int)gi;
       }
@@ -1180,6 +1352,7 @@ __device__ __forceinline__ void finish_one(const StepArgs& a, int d)
   bool last;
   const bool active = domain_dt(a, d, dt, dt_cfl, last);
   a.smax_bits[d] = 0ull;
+  if (a.slow32) a.slow32[d] = 0u;
   if (!active) return;
   if (a.fail[d]) { a.status[d] = a.fail[d]; return; }
   a.t[d] = last ? a.t_end : a.t[d] + dt;

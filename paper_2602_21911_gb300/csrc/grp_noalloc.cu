@@ -153,7 +153,9 @@ extern "C" int grp_step_noalloc(int system, double lambda, double gamma, int M, 
   a.dx = &w->dx; a.bc = &w->bc;
   a.avg = avg_in; a.avg_new = avg_out; a.ifc = iface_in; a.ifc_new = iface_out;
   a.flux = (double*)(base + OFF_FLUX);
-  a.pold = (double*)(base + OFF_POLD);
+  a.pold = nullptr;
+  a.rp32 = (float2*)(base + OFF_POLD);
+  a.gm1f = (float)a.ph.gm1; a.gammaf = (float)a.ph.gamma; a.h_gm1f = (float)a.ph.h_gm1;
   a.ds = (DomStep*)(base + OFF_DS);
   a.low = base + OFF_LOW; a.troubled = base + OFF_TROUBLED;
   a.t = &w->t; a.dt_prev = &w->dt_prev; a.nstep = &w->nstep; a.status = &w->status;
@@ -166,7 +168,7 @@ extern "C" int grp_step_noalloc(int system, double lambda, double gamma, int M, 
 
   // the flat step sequence of grp_step
   const bool euler = system == GRP_EULER_IDEAL;
-  if (euler) k_smax<<<nblk(N, 256), 256, 0, s>>>(a);
+  if (euler) k_speed<<<nblk(N, 256), 256, 0, s>>>(a);    // N <= SPEED_SMALL
   k_dt<<<1, 32, 0, s>>>(a);
   if (flux_dispatch(a, s) != cudaSuccess) return GRP_E_CUDA;
   if (euler) {
