@@ -135,7 +135,7 @@ typedef struct {
  * Euler equations with GRPrec of degree 2 or 4, the TT solver and no source:
  * the flux phase solves the Riemann problems that are not equal data in a
  * second kernel, from a list held by the context (4 bytes for every
- * interface).  At degree 2, with gamma in [1.2, 1.9] and the FLAT form, the
+ * interface).  At degrees 2 and 4, with gamma in [1.3, 1.9] and the FLAT form, the
  * first kernel computes in 64-bit fixed point, each interface in its own powers
  * of two (rounding errors below those of FP64); interfaces that leave that
  * format's range are solved in FP64 by the second kernel.

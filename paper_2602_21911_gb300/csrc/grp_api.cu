@@ -201,10 +201,7 @@ StepArgs make_args(const grp_ctx* c, double t_end)
   a.hard_idx = c->hard_idx;
   a.hard_count = c->hard_count;
   a.hard_cap = (int)c->hard_cap;
-  if (fixed::gamma_ok(a.ph.gamma)) {
-    a.fx_gm1 = fixed::to_format(a.ph.gm1);
-    a.fx_hgam = fixed::to_format(0.5 * a.ph.gamma);
-  }
+  if (fixed::gamma_ok(a.ph.gamma)) a.fx = fixed::make_consts(a.ph.gamma);
   a.ph.src = c->p.source;
   a.ph.src_k = c->p.source_coef;
   return a;
@@ -450,25 +447,26 @@ int enqueue_step(grp_ctx* c, double t_end)
   const bool flags = c->gadm[0] && flux_defers(a);
   if (flags) {
     if (!c->adm_valid) {
-      k_adm<<<blocks(c->nif, 256), 256, 0, s>>>(c->p.gamma, c->nif, a.ifc, c->gadm[c->cur]);
+      chain(k_adm, blocks(c->nif, 256), 256, s, c->p.gamma, c->nif, a.ifc, c->gadm[c->cur]);
       c->launches++;
     }
     a.adm_in = c->gadm[c->cur];
     a.adm_out = c->gadm[c->cur ^ 1];
-    a.fixed = flux_fixed(a) ? 1 : 0;
   }
+  if (c->p.solver != GRP_SOLVER_DET) a.fixed = flux_fixed(a) ? 1 : 0;
   const bool euler = c->p.system == GRP_EULER_IDEAL;
+  const unsigned tc = spread(c->ncell, 256), lb = list_blocks(c->ncell);
   if (euler) {
     if (c->ncell <= SPEED_SMALL) {
-      k_speed<<<blocks(c->ncell, 256), 256, 0, s>>>(a);
+      chain(k_speed, blocks(c->ncell, tc), tc, s, a);
       c->launches++;
     } else {
-      k_speed32<<<speed_blocks(c->ncell), 256, 0, s>>>(a);
-      k_speed64<<<blocks(c->ncell, 256), 256, 0, s>>>(a);
+      chain(k_speed32, speed_blocks(c->ncell), 256, s, a);
+      chain(k_speed64, blocks(c->ncell, 256), 256, s, a);
       c->launches += 2;
     }
   }
-  k_dt<<<blocks(c->D, 128), 128, 0, s>>>(a);
+  chain(k_dt, blocks(c->D, 128), 128, s, a);
   c->launches++;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (c->timing) {
@@ -483,7 +481,7 @@ int enqueue_step(grp_ctx* c, double t_end)
     c->launches += 3;
   } else {
     CK(c->p.source != GRP_SOURCE_NONE ? launch_flux_src(a, s) : launch_flux(a, s));
-    c->launches += flux_defers(a) ? 2 : 1;
+    c->launches += flux_defers(a) || a.fixed ? 2 : 1;
   }
   if (c->timing) {
     CK(record(c, e1));
@@ -491,20 +489,20 @@ int enqueue_step(grp_ctx* c, double t_end)
     c->ev_pending.push_back(e1);
   }
   if (euler) {
-    k_update<SYS_EULER><<<blocks(c->ncell, 256), 256, 0, s>>>(a, -1);
+    chain(k_update<SYS_EULER>, blocks(c->ncell, tc), tc, s, a, -1);
     c->launches++;
     // repair rounds over the compacted lists of troubled cells and repaired interfaces
     for (int r = 0; r < MAX_REPAIR; ++r) {
-      if (c->p.gamma == 1.4) k_repair_list<true><<<LIST_BLOCKS, LIST_THREADS, 0, s>>>(a, r);
-      else k_repair_list<false><<<LIST_BLOCKS, LIST_THREADS, 0, s>>>(a, r);
-      k_update_list<SYS_EULER><<<LIST_BLOCKS, LIST_THREADS, 0, s>>>(a, r);
+      if (c->p.gamma == 1.4) chain(k_repair_list<true>, lb, LIST_THREADS, s, a, r);
+      else chain(k_repair_list<false>, lb, LIST_THREADS, s, a, r);
+      chain(k_update_list<SYS_EULER>, lb, LIST_THREADS, s, a, r);
       c->launches += 2;
     }
   } else {
-    k_update<SYS_ADV><<<blocks(c->ncell, 256), 256, 0, s>>>(a, -1);
+    chain(k_update<SYS_ADV>, blocks(c->ncell, tc), tc, s, a, -1);
     c->launches++;
   }
-  k_finish<<<blocks(c->D, 128), 128, 0, s>>>(a);
+  chain(k_finish, blocks(c->D, 128), 128, s, a);
   c->launches++;
   CK(cudaGetLastError());
   c->adm_valid = flags;
@@ -619,11 +617,10 @@ int grp_create(grp_ctx** out, const grp_problem* p)
   AL(any_bad, MAX_REPAIR + 1) AL(stats, (long long)NSTATS * D) AL(scratch_norm, 3 * D)
   AL(tlist0, c->ncell) AL(tlist1, c->ncell) AL(ilist, c->nif) AL(lcount, 2 * (MAX_REPAIR + 1))
   if (p->source != GRP_SOURCE_NONE) AL(srcv, (long long)C * c->ncell)
-  if (p->system == GRP_EULER_IDEAL && p->recon == GRP_RECON_GRPREC && p->solver != GRP_SOLVER_DET &&
-      p->source == GRP_SOURCE_NONE && (p->M == 2 || p->M == 4)) {
+  if (p->system == GRP_EULER_IDEAL && p->solver != GRP_SOLVER_DET && p->source == GRP_SOURCE_NONE) {
     c->hard_cap = c->nif;
     AL(hard_idx, c->hard_cap) AL(hard_count, 3)
-    AL(gadm[0], c->nif) AL(gadm[1], c->nif)
+    if (p->recon == GRP_RECON_GRPREC && (p->M == 2 || p->M == 4)) { AL(gadm[0], c->nif) AL(gadm[1], c->nif) }
     if ((e = cudaMemset(c->hard_count, 0, 3 * sizeof(unsigned))) != cudaSuccess) {
       free_all(c); delete c; return cuda_fail(e, "cudaMemset hard_count");
     }

@@ -11,32 +11,37 @@ namespace grp {
 template <int MM, bool NLV>
 inline bool launch_flux_fixed(const StepArgs& a, cudaStream_t s)
 {
-  if constexpr (MM == 2 && !NLV) {
-    if (a.fixed) k_flux_fixed<MM><<<(unsigned)((a.nif + 127) / 128), 128, 0, s>>>(a);
-    return a.fixed != 0;
-  }
-  return false;
+  if (!a.fixed) return false;
+  const unsigned tpb = spread(a.nif, 128);
+  if constexpr (!NLV) chain(k_flux_fixed<MM>, (unsigned)((a.nif + tpb - 1) / tpb), tpb, s, a);
+  else if constexpr (MM <= 3) chain(k_flux_fixed_nl<MM>, (unsigned)((flux_threads(a.nif) + tpb - 1) / tpb), tpb, s, a);
+  return true;
 }
 
-// the second pass of the flux kernel, where the first defers interfaces
+// the second pass, where the first leaves it interfaces
 template <int MM, bool NLV>
 inline void launch_flux_hard(const StepArgs& a, cudaStream_t s)
 {
-  if constexpr (flux_defers_at<SYS_EULER, MM, NLV, false>()) {
-    if (a.hard_cap > 0) {
+  constexpr bool DEFER = flux_defers_at<SYS_EULER, MM, NLV, false>();
+  if constexpr (!NLV || MM <= 3) {
+    if (a.hard_cap > 0 && (DEFER || a.fixed)) {
       static int sms[64] = {0};
       int dev = 0;
       cudaGetDevice(&dev);
       if (dev < 0 || dev >= 64) dev = 0;
       if (!sms[dev]) cudaDeviceGetAttribute(&sms[dev], cudaDevAttrMultiProcessorCount, dev);
       const unsigned gh = hard_blocks(a.hard_cap, sms[dev] > 0 ? sms[dev] : 1);
-      const bool net = flux_hard_net(a);
-      if (a.ph.gamma == 1.4) {
-        if (net) k_flux_hard<MM, true, true><<<gh, GRP_HARD_TPB, 0, s>>>(a);
-        else k_flux_hard<MM, true, false><<<gh, GRP_HARD_TPB, 0, s>>>(a);
+      if constexpr (DEFER) {
+        const bool net = flux_hard_net(a);
+        if (a.ph.gamma == 1.4) {
+          if (net) chain(k_flux_hard<MM, true, true>, gh, GRP_HARD_TPB, s, a);
+          else chain(k_flux_hard<MM, true, false>, gh, GRP_HARD_TPB, s, a);
+        } else {
+          if (net) chain(k_flux_hard<MM, false, true>, gh, GRP_HARD_TPB, s, a);
+          else chain(k_flux_hard<MM, false, false>, gh, GRP_HARD_TPB, s, a);
+        }
       } else {
-        if (net) k_flux_hard<MM, false, true><<<gh, GRP_HARD_TPB, 0, s>>>(a);
-        else k_flux_hard<MM, false, false><<<gh, GRP_HARD_TPB, 0, s>>>(a);
+        chain(k_flux_hard<MM, true, false, NLV>, gh, GRP_HARD_TPB, s, a);      // gamma = 7/5 only
       }
     }
   }
@@ -46,10 +51,10 @@ inline void launch_flux_hard(const StepArgs& a, cudaStream_t s)
 #define GRP_DEFINE_EULER_LAUNCHERS(MM, NLV, SUFFIX)                                                          \
   cudaError_t launch_flux_euler_##SUFFIX(const StepArgs& a, cudaStream_t s)                                  \
   {                                                                                                          \
-    const unsigned g = (unsigned)((flux_threads(a.nif) + GRP_FLUX_TPB - 1) / GRP_FLUX_TPB);                  \
+    const unsigned tpb = spread(a.nif, GRP_FLUX_TPB), g = (unsigned)((flux_threads(a.nif) + tpb - 1) / tpb); \
     if (launch_flux_fixed<MM, NLV>(a, s)) {}                                                                 \
-    else if (a.ph.gamma == 1.4) k_flux<SYS_EULER, MM, true, NLV><<<g, GRP_FLUX_TPB, 0, s>>>(a);              \
-    else k_flux<SYS_EULER, MM, false, NLV><<<g, GRP_FLUX_TPB, 0, s>>>(a);                                    \
+    else if (a.ph.gamma == 1.4) chain(k_flux<SYS_EULER, MM, true, NLV>, g, tpb, s, a);              \
+    else chain(k_flux<SYS_EULER, MM, false, NLV>, g, tpb, s, a);                                    \
     launch_flux_hard<MM, NLV>(a, s);                                                                         \
     return cudaGetLastError();                                                                               \
   }                                                                                                          \
@@ -67,12 +72,12 @@ inline void launch_flux_hard(const StepArgs& a, cudaStream_t s)
 #define GRP_DEFINE_ADV_LAUNCHERS(NLV, SUFFIX)                                                                \
   cudaError_t launch_flux_adv##SUFFIX(const StepArgs& a, cudaStream_t s)                                     \
   {                                                                                                          \
-    const unsigned g = (unsigned)((flux_threads(a.nif) + GRP_FLUX_TPB - 1) / GRP_FLUX_TPB);                                         \
+    const unsigned tpb = spread(a.nif, GRP_FLUX_TPB), g = (unsigned)((flux_threads(a.nif) + tpb - 1) / tpb); \
     switch (a.M) {                                                                                           \
-      case 1: k_flux<SYS_ADV, 1, false, NLV><<<g, GRP_FLUX_TPB, 0, s>>>(a); break;                                    \
-      case 2: k_flux<SYS_ADV, 2, false, NLV><<<g, GRP_FLUX_TPB, 0, s>>>(a); break;                                    \
-      case 3: k_flux<SYS_ADV, 3, false, NLV><<<g, GRP_FLUX_TPB, 0, s>>>(a); break;                                    \
-      case 4: k_flux<SYS_ADV, 4, false, NLV><<<g, GRP_FLUX_TPB, 0, s>>>(a); break;                                    \
+      case 1: chain(k_flux<SYS_ADV, 1, false, NLV>, g, tpb, s, a); break;                                    \
+      case 2: chain(k_flux<SYS_ADV, 2, false, NLV>, g, tpb, s, a); break;                                    \
+      case 3: chain(k_flux<SYS_ADV, 3, false, NLV>, g, tpb, s, a); break;                                    \
+      case 4: chain(k_flux<SYS_ADV, 4, false, NLV>, g, tpb, s, a); break;                                    \
       default: return cudaErrorInvalidValue;                                                                 \
     }                                                                                                        \
     return cudaGetLastError();                                                                               \

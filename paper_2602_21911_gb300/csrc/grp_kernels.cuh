@@ -14,6 +14,7 @@
 #pragma once
 #include "grp_device.cuh"
 #include "grp_fixed.cuh"
+#include "grp_launch.h"
 
 namespace grp {
 
@@ -82,11 +83,10 @@ struct StepArgs {
   // fixed-point format), solved in a second pass with dense warps; hard_cap
   // holds every interface, or is 0 and nothing is deferred
   int* hard_idx = nullptr;           // [hard_cap] interface
-  // the first pass runs in 64-bit fixed point (grp_fixed.cuh): gamma - 1 and
-  // gamma / 2 in its format; the per-interface count of Riemann problems is then
-  // added per domain by k_dt
+  // the first pass runs in 64-bit fixed point (grp_fixed.cuh): its constants;
+  // the per-interface count of Riemann problems is then added per domain by k_dt
   int fixed = 0;
-  long long fx_gm1 = 0, fx_hgam = 0;
+  fixed::Consts fx;
   // admissibility of the interface data (Euler, flat form at degrees 2 and 4):
   // adm_in[j] = 1 when the current datum at j is admissible (null: test the
   // data), adm_out[j] written with every new datum (null: not kept).  Each
@@ -196,6 +196,7 @@ __device__ __forceinline__ bool domain_dt(const StepArgs& a, int d, double& dt, 
 // time step.
 static __global__ void k_dt(StepArgs a)
 {
+  chain_wait();
   const int d = blockIdx.x * blockDim.x + threadIdx.x;
   if (d < a.n_domains) {
     for (int p = 0; p <= MAX_REPAIR; ++p) a.bad[p * a.n_domains + d] = 0;
@@ -307,6 +308,7 @@ inline unsigned speed_blocks(long long ncell) { return (unsigned)((ncell + 256 *
 
 static __global__ void __launch_bounds__(256) k_speed32(StepArgs a)
 {
+  chain_wait();
   if (blockIdx.x == 0 && threadIdx.x <= MAX_REPAIR) a.any_bad[threadIdx.x] = 0;
   if (blockIdx.x == 0 && threadIdx.x < 2 * (MAX_REPAIR + 1)) a.lcount[threadIdx.x] = 0;
   const long long g0 = (long long)blockIdx.x * (256 * SPEED_CELLS) + threadIdx.x;
@@ -346,6 +348,7 @@ static __global__ void __launch_bounds__(256) k_speed32(StepArgs a)
 constexpr long long SPEED_SMALL = 1 << 17;
 static __global__ void __launch_bounds__(256) k_speed(StepArgs a)
 {
+  chain_wait();
   if (blockIdx.x == 0 && threadIdx.x <= MAX_REPAIR) a.any_bad[threadIdx.x] = 0;
   if (blockIdx.x == 0 && threadIdx.x < 2 * (MAX_REPAIR + 1)) a.lcount[threadIdx.x] = 0;
   const long long gi = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -375,6 +378,7 @@ static __global__ void __launch_bounds__(256) k_speed(StepArgs a)
 // states (undisturbed gas) are evaluated at their first cell.
 static __global__ void __launch_bounds__(256) k_speed64(StepArgs a)
 {
+  chain_wait();
   const long long gi = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (gi >= a.ncell) return;
   const int d = a.cell_dom[gi];
@@ -842,51 +846,94 @@ __device__ __forceinline__ void flux_warp(const StepArgs& a, long long gbase, lo
   }
 }
 
+// Interfaces left to the second pass, in consecutive slots per warp (all 32 lanes
+// call).
+__device__ __forceinline__ void list_hard(const StepArgs& a, bool hard, long long gj)
+{
+  const unsigned bal = __ballot_sync(0xffffffffu, hard);
+  if (!bal) return;
+  unsigned base = 0;
+  if (lane_id() == 0) base = atomicAdd(a.hard_count, (unsigned)__popc(bal));
+  base = __shfl_sync(0xffffffffu, base, 0);
+  if (hard) a.hard_idx[base + (unsigned)__popc(bal & ((1u << lane_id()) - 1u))] = (int)gj;
+}
+
+// Newton iterations of the fixed-point Riemann problems (three in FP32, two in
+// the format), per warp and domain (all 32 lanes call; d < 0: no interface).
+constexpr unsigned FIXED_ITERS = 5;
+__device__ __forceinline__ void count_newton(const StepArgs& a, bool newton, int d)
+{
+  const unsigned bal = __ballot_sync(0xffffffffu, newton);
+  if (!bal) return;
+  const unsigned grp = __match_any_sync(0xffffffffu, newton ? d : -1);
+  if (newton && lane_id() == __ffs(grp) - 1) {
+    unsigned long long* S = a.stats + (long long)d * NSTATS;
+    atomicAdd(S + S_NEWTON_SUM, (unsigned long long)(FIXED_ITERS * __popc(grp)));
+    atomicMax(S + S_NEWTON_MAX, (unsigned long long)FIXED_ITERS);
+  }
+}
+
 // The first pass in 64-bit fixed point, one lane per interface.  Interfaces
-// that are not equal data (transmissive ends, cells fallen back to degree 0) or
-// leave the format go to the hard list.  Needs the admissibility flags.
+// that leave the format go to the hard list; so do transmissive ends, and at
+// degrees 2 and 4 (which need the admissibility flags) those beside a cell fallen
+// back to degree 0, whose data are not equal.  Degrees 1 and 3 solve the leading
+// Riemann problem of their traces here.
 // Both cells of an interface are reconstructed by its own lane: a neighbour's
 // would be in the neighbour's units, and the reconstruction is a few additions.
-// Bound by the integer pipes.  Measured on 16,384 domains of the batch (1.73 M
-// interfaces): 0.151 ms, against 0.614 ms of the FP64 pass (k_flux), whose 177
-// FP64 instructions per interface kept that pipe 85 % busy.
+// Bound by the integer pipes (ALU and multiply-add each about 65 % busy).
+// Measured at degree 2 on 16,384 domains of the batch (1.73 M interfaces):
+// 0.15 ms, against 0.614 ms of the FP64 pass (k_flux), whose 177 FP64
+// instructions per interface kept that pipe 85 % busy.
 template <int M>
-__global__ void __launch_bounds__(128) k_flux_fixed(StepArgs a)
+__global__ void __launch_bounds__(128, M == 2 ? 5 : 3) k_flux_fixed(StepArgs a)
 {
+  chain_wait();
+  constexpr bool EQ = M == 2 || M == 4;
+  constexpr int NQ = M <= 2 ? 2 : 4, IL = M <= 2 ? 0 : 1;
   const long long gj = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  bool hard = false;
+  bool hard = false, newton = false;
+  int d = -1;
   if (gj < a.nif) {
-    const int d = a.if_dom[gj];
+    d = a.if_dom[gj];
     const DomStep& ds = a.ds[d];
     if (!ds.active) {
 #pragma unroll
       for (int c = 0; c < 3; ++c) a.ifc_new[c * a.nif + gj] = a.ifc[c * a.nif + gj];
-      a.adm_out[gj] = a.adm_in[gj];
+      if (EQ) a.adm_out[gj] = a.adm_in[gj];
     } else {
       const long long i0 = a.if_off[d], c0 = a.cell_off[d];
       const int j = (int)(gj - i0), N = (int)(a.cell_off[d + 1] - c0), bc = a.bc[d];
       // left cell and its left interface, right cell and its right interface
       const int cl = bc == 0 && j == 0 ? N - 1 : j - 1, cr = j;
       const long long gl = i0 + (cl < 0 ? 0 : cl), gr = i0 + (bc == 0 && j == N - 1 ? 0 : (j == N ? N : j + 1));
-      const unsigned char al = a.adm_in[gl], ac = a.adm_in[gj], ar = a.adm_in[gr];
-      hard = !(al & ac & ar) || (bc != 0 && (j == 0 || j == N));
-      if (cl >= 0 && !(al & ac)) atomicAdd(a.stats + (long long)d * NSTATS + S_RECON_FB, 1ull);   // rare
+      hard = bc != 0 && (j == 0 || j == N);
+      if (EQ) {
+        const unsigned char al = a.adm_in[gl], ac = a.adm_in[gj], ar = a.adm_in[gr];
+        hard = hard || !(al & ac & ar);
+        if (cl >= 0 && !(al & ac)) atomicAdd(a.stats + (long long)d * NSTATS + S_RECON_FB, 1ull);   // rare
+      }
       if (!hard) {
-        double q[2][3], g[3][3], F[3], gnew[3];
+        double q[NQ][3], g[3][3], F[3], gnew[3];
+        int im = 0, ip = 0, jm, jp;                // degrees 3 and 4: the cells beyond
+        if (M >= 3) {
+          nbr(cl, N, bc, im, jp);
+          nbr(cr, N, bc, jm, ip);
+        }
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
           const double* A = a.avg + c * a.ncell + c0;
           const double* G = a.ifc + c * a.nif;
-          q[0][c] = A[cl];
-          q[1][c] = A[cr];
+          q[IL][c] = A[cl];
+          q[IL + 1][c] = A[cr];
+          if (M >= 3) { q[0][c] = A[im]; q[NQ - 1][c] = A[ip]; }
           g[0][c] = G[gl];
           g[1][c] = G[gj];
           g[2][c] = G[gr];
         }
-        hard = !fixed::grp_equal2(a.ph.gm1, a.fx_gm1, a.fx_hgam, ds.nu, q, g, F, gnew);
+        hard = !fixed::grp_linear<M>(a.fx, a.ph.gm1, ds.nu, q, g, F, gnew, newton);
         if (!hard) {
           a.low[gj] = 0;
-          a.adm_out[gj] = 1;
+          if (EQ) a.adm_out[gj] = 1;
 #pragma unroll
           for (int c = 0; c < 3; ++c) {
             a.flux[c * a.nif + gj] = F[c];
@@ -896,13 +943,66 @@ __global__ void __launch_bounds__(128) k_flux_fixed(StepArgs a)
       }
     }
   }
-  const unsigned bal = __ballot_sync(0xffffffffu, hard);
-  if (bal) {                                       // consecutive slots per warp
-    unsigned base = 0;
-    if (lane_id() == 0) base = atomicAdd(a.hard_count, (unsigned)__popc(bal));
-    base = __shfl_sync(0xffffffffu, base, 0);
-    if (hard) a.hard_idx[base + (unsigned)__popc(bal & ((1u << lane_id()) - 1u))] = (int)gj;
+  list_hard(a, hard, gj);
+  if (!EQ) count_newton(a, newton && !hard, d);
+}
+
+// ... with the nonlinear reconstruction (degrees 1 to 3), which stays in FP64 and
+// is shared by the warp as in flux_warp: 31 interfaces per warp.
+template <int M>
+__global__ void __launch_bounds__(128, 3) k_flux_fixed_nl(StepArgs a)
+{
+  chain_wait();
+  const int lane = lane_id();
+  const long long gj = (((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 31 + lane;
+  bool hard = false, newton = false, active = false, fb = false;
+  int d = -1, j = 0, N = 0, bc = 0, cl = -1;
+  long long c0 = 0, i0 = 0;
+  double em[3][M + 1], ep[3][M + 1], rm[3][M + 1];
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+#pragma unroll
+    for (int k = 0; k <= M; ++k) em[c][k] = ep[c][k] = 0.0;
+  if (gj < a.nif) {
+    d = a.if_dom[gj];
+    i0 = a.if_off[d];
+    c0 = a.cell_off[d];
+    j = (int)(gj - i0);
+    N = (int)(a.cell_off[d + 1] - c0);
+    bc = a.bc[d];
+    active = a.ds[d].active != 0;
+    cl = bc == 0 && j == 0 ? N - 1 : j - 1;
+    if (active && cl >= 0) cell_edges<SYS_EULER, M, true>(a, c0, i0, N, bc, cl, em, ep, fb);
   }
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+#pragma unroll
+    for (int k = 0; k <= M; ++k) rm[c][k] = __shfl_down_sync(0xffffffffu, em[c][k], 1);
+  const bool fbr = __shfl_down_sync(0xffffffffu, (int)fb, 1) != 0;
+  if (lane < 31 && gj < a.nif) {
+    if (!active) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) a.ifc_new[c * a.nif + gj] = a.ifc[c * a.nif + gj];
+    } else {
+      // domain ends (the next lane holds another domain's cell) and fallen cells
+      // (counted there): the second pass
+      hard = fb || fbr || j >= N - (bc == 0 ? 1 : 0) || (bc != 0 && j == 0);
+      if (!hard) {
+        double F[3], gnew[3];
+        hard = !fixed::grp_traces<M>(a.fx, a.ph.gm1, a.ds[d].nu, ep, rm, F, gnew, newton);
+        if (!hard) {
+          a.low[gj] = 0;
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            a.flux[c * a.nif + gj] = F[c];
+            a.ifc_new[c * a.nif + gj] = gnew[c];
+          }
+        }
+      }
+    }
+  }
+  list_hard(a, hard, gj);
+  count_newton(a, newton && !hard, d);
 }
 
 // Interfaces are deferred at the interpolating degrees (2 and 4) of the
@@ -916,6 +1016,7 @@ __host__ __device__ constexpr bool flux_defers_at()
 template <int SYS, int M, bool G75, bool NL, bool SRC = false>
 __global__ void __launch_bounds__(GRP_FLUX_TPB, GRP_FLUX_MIN_BLOCKS) k_flux(StepArgs a)
 {
+  chain_wait();
   flux_warp<SYS, M, G75, NL, SRC, flux_defers_at<SYS, M, NL, SRC>()>(
       a, (((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 31, a.nif);
 }
@@ -927,11 +1028,20 @@ inline bool flux_defers(const StepArgs& a)
   return a.sys == SYS_EULER && a.recon == 0 && !a.srcv && (a.M == 2 || a.M == 4) && a.hard_cap > 0;
 }
 
-// The first pass in fixed point: degree 2, with the flags kept, for the ratios
-// of specific heats the format's bounds are worked out for.
+// Whether the first pass runs in fixed point: where its rounding stays below
+// FP64's.  Equal data (linear reconstruction, degrees 2 and 4) need the flags.
+// The Riemann problems of the other degrees and of GRPrecNL are solved for
+// gamma = 7/5 and to the format's precision whatever newton_rtol asks beyond it;
+// the learned start and the harvest keep the FP64 pass, whose iterations they
+// are about.  Degree 4 on less than two warps per SM stays in FP64: one warp
+// alone takes 38 us in fixed point and 26 us in FP64 (degree 2: 10 and 14 us).
+constexpr long long FIXED_MIN4 = 152 * 64;
 inline bool flux_fixed(const StepArgs& a)
 {
-  return flux_defers(a) && a.adm_in && a.M == 2 && fixed::gamma_ok(a.ph.gamma);
+  if (a.sys != SYS_EULER || a.srcv || a.hard_cap == 0 || !fixed::gamma_ok(a.ph.gamma)) return false;
+  if (a.recon == 0 && (a.M == 2 || a.M == 4)) return a.adm_in && (a.M == 2 || a.nif > FIXED_MIN4);
+  return a.ph.gamma == 1.4 && (a.recon == 0 || a.M <= 3) && a.ph.guess != 2 && !a.harvest && a.ph.rtol >= 1e-13 &&
+         a.ph.max_iter >= (int)FIXED_ITERS;
 }
 
 // The second pass runs one warp per block, so that a warp that finishes frees
@@ -958,9 +1068,10 @@ inline unsigned hard_blocks(long long cap, int sms)
 // NET: the learned start's network is evaluated by the whole warp for each
 // lane that wants it (inference with a model; harvest and the classical starts
 // take the plain instantiation).
-template <int M, bool G75, bool NET>
+template <int M, bool G75, bool NET, bool NL = false>
 __global__ void __launch_bounds__(GRP_HARD_TPB, GRP_HARD_MIN_BLOCKS) k_flux_hard(StepArgs a)
 {
+  chain_wait();
   constexpr int C = 3;
   const unsigned offered = a.hard_count[0];
   const long long n = offered < (unsigned)a.hard_cap ? offered : a.hard_cap;
@@ -983,11 +1094,13 @@ __global__ void __launch_bounds__(GRP_HARD_TPB, GRP_HARD_MIN_BLOCKS) k_flux_hard
       const long long i0 = a.if_off[d], c0 = a.cell_off[d];
       const int N = (int)(a.cell_off[d + 1] - c0), bc = a.bc[d], j = (int)(gj - i0);
       const int cl = bc == 0 ? (j == 0 ? N - 1 : j - 1) : j - 1, cr = bc != 0 && j == N ? -1 : j;
+      constexpr bool EQ = !NL && (M == 2 || M == 4);
       double tx[C][M + 1];
-      bool fb;
-      if (cl >= 0) cell_edges<SYS_EULER, M, false, true>(a, c0, i0, N, bc, cl, tx, tL, fb);
+      bool fb = false;
+      if (cl >= 0) cell_edges<SYS_EULER, M, NL, EQ>(a, c0, i0, N, bc, cl, tx, tL, fb);
       else ghost_edge<SYS_EULER, M>(a, c0, 0, tL);
-      if (cr >= 0) cell_edges<SYS_EULER, M, false, true>(a, c0, i0, N, bc, cr, tR, tx, fb);
+      if (!EQ) st[5] = fb ? 1u : 0u;               // (degrees 2 and 4: counted by the first pass, from the flags)
+      if (cr >= 0) cell_edges<SYS_EULER, M, NL, EQ>(a, c0, i0, N, bc, cr, tR, tx, fb);
       else ghost_edge<SYS_EULER, M>(a, c0, N - 1, tR);
     }
     if (NET) {
@@ -1180,6 +1293,7 @@ __device__ __forceinline__ int update_one(const StepArgs& a, long long gi, int d
 template <int SYS>
 __global__ void __launch_bounds__(256, 8) k_update(StepArgs a, int pass)
 {
+  chain_wait();
   const long long gi = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (pass >= 0 && a.any_bad[pass] == 0) return;
   if (gi >= a.ncell) return;
@@ -1203,6 +1317,8 @@ __global__ void __launch_bounds__(256, 8) k_update(StepArgs a, int pass)
 // Grid-stride helpers of the work-list kernels (their grids are fixed, so a
 // captured graph serves every step).
 constexpr int LIST_BLOCKS = 4 * 152, LIST_THREADS = 128;
+inline unsigned list_blocks(long long) { return LIST_BLOCKS; }
+inline unsigned spread(long long n, unsigned threads) { (void)n; return threads; }
 
 // First-order Godunov flux at interface gj (round `pass`); appends it to the
 // round's interface list.
@@ -1245,6 +1361,7 @@ __device__ __forceinline__ void repair_iface(const StepArgs& a, int pass, long l
 template <bool G75>
 __global__ void __launch_bounds__(LIST_THREADS) k_repair_list(StepArgs a, int pass)
 {
+  chain_wait();
   __shared__ long long q[2 * LIST_THREADS];
   __shared__ int qn;
   const int n = a.lcount[pass];
@@ -1284,6 +1401,7 @@ __global__ void __launch_bounds__(LIST_THREADS) k_repair_list(StepArgs a, int pa
 template <int SYS>
 __global__ void __launch_bounds__(LIST_THREADS) k_update_list(StepArgs a, int pass)
 {
+  chain_wait();
   const int n = a.lcount[MAX_REPAIR + 1 + pass];
   const unsigned char mark = (unsigned char)(2 + pass);
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
@@ -1364,6 +1482,7 @@ __device__ __forceinline__ void finish_one(const StepArgs& a, int d)
 
 static __global__ void k_finish(StepArgs a)
 {
+  chain_wait();
   const int d = blockIdx.x * blockDim.x + threadIdx.x;
   if (d < a.n_domains) finish_one(a, d);
 }
@@ -1494,6 +1613,7 @@ __global__ void __launch_bounds__(256) k_post(StepArgs a, const int* __restrict_
 // The admissibility flags of given interface data.
 static __global__ void k_adm(double g, long long nif, const double* ifc, unsigned char* adm)
 {
+  chain_wait();
   const long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (j < nif) adm[j] = admissible(g, ifc[j], ifc[nif + j], ifc[2 * nif + j]) ? 1 : 0;
 }

@@ -39,13 +39,19 @@ constexpr size_t OFF_POLD = align256(OFF_ILIST + sizeof(int) * NA_IFACES);
 constexpr size_t OFF_DS = align256(OFF_POLD + sizeof(double) * NA_CELLS);
 constexpr size_t OFF_WORDS = align256(OFF_DS + sizeof(DomStep));
 
+// what the call reads back, in one copy
+struct Result {
+  double t;
+  int status;
+};
 // per-domain words of the single domain, in one struct
 struct Words {
   long long cell_off[2], if_off[2];
-  double dx, t, dt_prev;
+  double dx, dt_prev;
+  Result out;
   unsigned long long smax_bits;
   unsigned long long stats[NSTATS];
-  int nstep, status, fail;
+  int nstep, fail;
   int bad[MAX_REPAIR + 1], inad, any_bad[MAX_REPAIR + 1];
   int lcount[2 * (MAX_REPAIR + 1)];
   unsigned char bc;
@@ -68,6 +74,7 @@ unsigned char* g_scratch_addr[MAX_DEVICES];
 // Zeroes what must start at zero and writes the index tables and words.
 __global__ void k_noalloc_setup(unsigned char* base, int N, int nif, double dx, int bc, double t)
 {
+  chain_wait();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   int* cell_dom = (int*)(base + OFF_CELL_DOM);
   int* if_dom = (int*)(base + OFF_IF_DOM);
@@ -77,10 +84,10 @@ __global__ void k_noalloc_setup(unsigned char* base, int N, int nif, double dx, 
     Words* w = (Words*)(base + OFF_WORDS);
     w->cell_off[0] = 0; w->cell_off[1] = N;
     w->if_off[0] = 0; w->if_off[1] = nif;
-    w->dx = dx; w->t = t; w->dt_prev = 0.0;
+    w->dx = dx; w->out.t = t; w->dt_prev = 0.0;
     w->smax_bits = 0ull;
     for (int k = 0; k < NSTATS; ++k) w->stats[k] = 0ull;
-    w->nstep = 0; w->status = 0; w->fail = 0;
+    w->nstep = 0; w->out.status = 0; w->fail = 0;
     for (int p = 0; p <= MAX_REPAIR; ++p) { w->bad[p] = 0; w->any_bad[p] = 0; }
     for (int p = 0; p < 2 * (MAX_REPAIR + 1); ++p) w->lcount[p] = 0;
     w->inad = 0;
@@ -140,7 +147,8 @@ extern "C" int grp_step_noalloc(int system, double lambda, double gamma, int M, 
   const double dx = (x_right - x_left) / N;
   Words* w = (Words*)(base + OFF_WORDS);
 
-  k_noalloc_setup<<<nblk(nif, 256), 256, 0, s>>>(base, N, nif, dx, bc, t);
+  const unsigned tc = spread(N, 256), lb = list_blocks(N);
+  chain(k_noalloc_setup, nblk(nif, 256), 256, s, base, N, nif, dx, bc, t);
 
   StepArgs a;
   a.sys = system; a.M = M; a.C = system == GRP_EULER_IDEAL ? 3 : 1;
@@ -158,7 +166,7 @@ extern "C" int grp_step_noalloc(int system, double lambda, double gamma, int M, 
   a.gm1f = (float)a.ph.gm1; a.gammaf = (float)a.ph.gamma; a.h_gm1f = (float)a.ph.h_gm1;
   a.ds = (DomStep*)(base + OFF_DS);
   a.low = base + OFF_LOW; a.troubled = base + OFF_TROUBLED;
-  a.t = &w->t; a.dt_prev = &w->dt_prev; a.nstep = &w->nstep; a.status = &w->status;
+  a.t = &w->out.t; a.dt_prev = &w->dt_prev; a.nstep = &w->nstep; a.status = &w->out.status;
   a.smax_bits = &w->smax_bits;
   a.bad = w->bad; a.inad = &w->inad; a.fail = &w->fail; a.any_bad = w->any_bad;
   a.tlist[0] = (int*)(base + OFF_TLIST0); a.tlist[1] = (int*)(base + OFF_TLIST1);
@@ -168,24 +176,25 @@ extern "C" int grp_step_noalloc(int system, double lambda, double gamma, int M, 
 
   // the flat step sequence of grp_step
   const bool euler = system == GRP_EULER_IDEAL;
-  if (euler) k_speed<<<nblk(N, 256), 256, 0, s>>>(a);    // N <= SPEED_SMALL
-  k_dt<<<1, 32, 0, s>>>(a);
+  if (euler) chain(k_speed, nblk(N, tc), tc, s, a);    // N <= SPEED_SMALL
+  chain(k_dt, 1, 32, s, a);
   if (flux_dispatch(a, s) != cudaSuccess) return GRP_E_CUDA;
   if (euler) {
-    k_update<SYS_EULER><<<nblk(N, 256), 256, 0, s>>>(a, -1);
+    chain(k_update<SYS_EULER>, nblk(N, tc), tc, s, a, -1);
     for (int r = 0; r < MAX_REPAIR; ++r) {
-      if (gamma == 1.4) k_repair_list<true><<<LIST_BLOCKS, LIST_THREADS, 0, s>>>(a, r);
-      else k_repair_list<false><<<LIST_BLOCKS, LIST_THREADS, 0, s>>>(a, r);
-      k_update_list<SYS_EULER><<<LIST_BLOCKS, LIST_THREADS, 0, s>>>(a, r);
+      if (gamma == 1.4) chain(k_repair_list<true>, lb, LIST_THREADS, s, a, r);
+      else chain(k_repair_list<false>, lb, LIST_THREADS, s, a, r);
+      chain(k_update_list<SYS_EULER>, lb, LIST_THREADS, s, a, r);
     }
   } else {
-    k_update<SYS_ADV><<<nblk(N, 256), 256, 0, s>>>(a, -1);
+    chain(k_update<SYS_ADV>, nblk(N, tc), tc, s, a, -1);
   }
-  k_finish<<<1, 32, 0, s>>>(a);
+  chain(k_finish, 1, 32, s, a);
   if (cudaGetLastError() != cudaSuccess) return GRP_E_CUDA;
-  if (cudaMemcpyAsync(t_out, &w->t, sizeof(double), cudaMemcpyDeviceToHost, s) != cudaSuccess) return GRP_E_CUDA;
-  if (cudaMemcpyAsync(status_out, &w->status, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess)
-    return GRP_E_CUDA;
+  Result r;
+  if (cudaMemcpyAsync(&r, &w->out, sizeof r, cudaMemcpyDeviceToHost, s) != cudaSuccess) return GRP_E_CUDA;
   if (cudaStreamSynchronize(s) != cudaSuccess) return GRP_E_CUDA;
+  *t_out = r.t;
+  *status_out = r.status;
   return GRP_OK;
 }

@@ -1,4 +1,4 @@
-"""The fixed-point GRP of the flux kernel's first pass (degree 2, equal data)
+"""The fixed-point GRP of the flux kernel's first pass (degrees 2 and 4, equal data)
 on the host: its errors against quad precision are below those of the FP64
 path over the ratios of specific heats, slopes and Mach numbers it accepts, and
 what it must leave to the general path (sonic fields, cut series) it leaves."""
@@ -28,16 +28,17 @@ def lines(tmp_path_factory):
 
 
 def test_errors_are_below_the_fp64_path(lines):
-    assert len(lines) == 20
-    for gamma, slope, share, rms, mx, rms64, mx64, wrong in lines:
+    assert len(lines) == 65
+    for degree, traces, gamma, slope, share, rms, mx, rms64, mx64, wrong in lines:
         # rms below FP64's; a single result is rounded to a double of up to
         # twice its unit (2^-52 of rho a^2 / (gamma (gamma - 1)))
-        assert rms <= rms64, (gamma, slope, rms, rms64)
-        assert mx <= max(mx64, 2.0 ** -52 * 2.0 / (gamma * (gamma - 1.0))), (gamma, slope, mx, mx64)
+        assert rms <= rms64, (degree, gamma, slope, rms, rms64)
+        assert mx <= max(mx64, 2.0 ** -52 * 2.0 / (gamma * (gamma - 1.0))), (degree, gamma, slope, mx, mx64)
 
 
 def test_what_is_accepted(lines):
-    for gamma, slope, share, rms, mx, rms64, mx64, wrong in lines:
-        assert wrong == 0, (gamma, slope)
-        if slope <= 0.3 and 1.3 <= gamma:
-            assert share >= 0.99, (gamma, slope, share)
+    for degree, traces, gamma, slope, share, rms, mx, rms64, mx64, wrong in lines:
+        assert wrong == 0, (degree, gamma, slope)
+        if 1.3 <= gamma and slope <= (0.3 if degree == 2 else 0.05):
+            # (with a leading Riemann problem, the tenth or so beyond Mach 2 is left)
+            assert share >= (0.99 if degree in (2, 4) and not traces else 0.9), (degree, gamma, slope, share)
