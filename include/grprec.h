@@ -132,13 +132,16 @@ typedef struct {
 /*
  * Create a context for the problem *p (copied; the arrays are read during the
  * call only).  Allocates the device state.  *out receives the context.
- * Euler equations with GRPrec of degree 2 or 4, the TT solver and no source:
- * the flux phase solves the Riemann problems that are not equal data in a
- * second kernel, from a list held by the context (4 bytes for every
- * interface).  At degrees 2 and 4, with gamma in [1.3, 1.9] and the FLAT form, the
- * first kernel computes in 64-bit fixed point, each interface in its own powers
- * of two (rounding errors below those of FP64); interfaces that leave that
- * format's range are solved in FP64 by the second kernel.
+ * Euler equations, the TT solver, no source and the FLAT form: the flux phase
+ * solves interfaces that the first kernel leaves (degrees 2 and 4: those whose
+ * Riemann problem is not one of equal data) in a second kernel, from a list held
+ * by the context (4 bytes for every interface).  On all but small grids the first
+ * kernel computes in 64-bit fixed point, each interface in its own powers of two
+ * (rounding errors below those of FP64): at degrees 2 and 4 with gamma in [1.3,
+ * 1.9], at degrees 1 and 3 and for GRPrecNL up to degree 3 with gamma = 7/5 and a
+ * classical Newton start, where a Riemann problem counts 5 iterations in the
+ * statistics; interfaces that leave that format's range are solved in FP64 by the
+ * second kernel.
  * Errors: GRP_E_INVALID_ARG for any field outside its range, GRP_E_CUDA.
  */
 int grp_create(grp_ctx **out, const grp_problem *p);

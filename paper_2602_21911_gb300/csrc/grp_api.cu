@@ -35,7 +35,9 @@ struct grp_ctx {
   double* flux = nullptr;
   double* pold = nullptr;        // pressure of the current averages (S_max pass)
   unsigned* slow32 = nullptr;    // per-domain FP32 lower bound of S_max (flat form)
-  DomStep* ds = nullptr;         // per-domain time step of the current step
+  DomStep* ds = nullptr;         // per-domain time steps: of the current step, and (advection) of the next
+  bool ds_ready = false;         // advection: ds of buffer cur is that of the current state ...
+  unsigned long long ds_t_end = 0;   // ... for this t_end (bits)
   double* det_ed = nullptr;      // DET: evolved edge values of every cell
   double* srcv = nullptr;        // numerical source of every cell (source terms only)
   int* hard_idx = nullptr;       // flux kernel's deferred interfaces, and its counters
@@ -80,6 +82,7 @@ struct grp_ctx {
     int start_cur = 0;
     bool smax_ready = false;
     bool adm_valid = false, adm_end = false;   // flags valid at the graph's start and end
+    bool ds_ready = false, ds_end = false;     // time steps ready at the graph's start and end
     unsigned long long t_end_bits = 0;
     int steps = 0;
     int cur_end = 0;                 // buffer parity after the graph
@@ -281,6 +284,7 @@ int build_groups(grp_ctx* c)
 // nsteps steps of the persistent batched kernel in one launch
 int enqueue_batch(grp_ctx* c, int nsteps, double t_end)
 {
+  c->ds_ready = false;
   c->adm_valid = false;               // this form keeps no admissibility flags
   if (!c->grp) { const int rc = build_groups(c); if (rc) return rc; }
   c->smax_ready = false;
@@ -310,6 +314,7 @@ int enqueue_batch(grp_ctx* c, int nsteps, double t_end)
 // one step in the split form: grid-wide k_flux, then k_post per domain group
 int enqueue_split(grp_ctx* c, double t_end)
 {
+  c->ds_ready = false;
   c->adm_valid = false;               // this form keeps no admissibility flags
   if (!c->grp) { const int rc = build_groups(c); if (rc) return rc; }
   const StepArgs a = make_args(c, t_end);
@@ -394,6 +399,7 @@ int build_tiles(grp_ctx* c)
 // steps_per_launch steps of every domain in one tile launch (t_end = inf)
 int enqueue_tiled(grp_ctx* c)
 {
+  c->ds_ready = false;
   c->adm_valid = false;               // this form keeps no admissibility flags
   if (!c->tiles) { const int rc = build_tiles(c); if (rc) return rc; }
   c->smax_ready = false;
@@ -437,17 +443,58 @@ int enqueue_tiled(grp_ctx* c)
   return GRP_OK;
 }
 
+unsigned long long bits_of(double x)
+{
+  unsigned long long b;
+  memcpy(&b, &x, sizeof b);
+  return b;
+}
+
+// one advection step: one launch, after a first one that forms the time steps
+int enqueue_advection(grp_ctx* c, StepArgs a)
+{
+  cudaStream_t s = c->stream;
+  a.ds = c->ds + (long long)c->cur * c->D;
+  if (!c->ds_ready || c->ds_t_end != bits_of(a.t_end)) {
+    k_dt<<<blocks(c->D, 128), 128, 0, s>>>(a);
+    c->launches++;
+  }
+  cudaEvent_t e0 = nullptr, e1 = nullptr;
+  if (c->timing) {
+    for (cudaEvent_t* e : {&e0, &e1}) {
+      if (!c->ev_free.empty()) { *e = c->ev_free.back(); c->ev_free.pop_back(); }
+      else CK(cudaEventCreate(e));
+    }
+    CK(record(c, e0));
+  }
+  DomStep* next = c->ds + (long long)(c->cur ^ 1) * c->D;
+  CK(a.recon == GRP_RECON_GRPRECNL ? launch_adv_step_nl(a, next, s) : launch_adv_step(a, next, s));
+  c->launches++;
+  if (c->timing) {
+    CK(record(c, e1));
+    c->ev_pending.push_back(e0);
+    c->ev_pending.push_back(e1);
+  }
+  c->ds_ready = true;
+  c->ds_t_end = bits_of(a.t_end);
+  c->cur ^= 1;
+  c->host_steps += 1;
+  return GRP_OK;
+}
+
 int enqueue_step(grp_ctx* c, double t_end)
 {
   c->smax_ready = false;
   StepArgs a = make_args(c, t_end);
   cudaStream_t s = c->stream;
+  if (c->p.system == GRP_ADVECTION && c->p.solver == GRP_SOLVER_TT && c->p.source == GRP_SOURCE_NONE)
+    return enqueue_advection(c, a);
   // the flat flux kernel at degrees 2 and 4 keeps the interface data's
   // admissibility flags; after a step of another form they are formed anew
   const bool flags = c->gadm[0] && flux_defers(a);
   if (flags) {
     if (!c->adm_valid) {
-      chain(k_adm, blocks(c->nif, 256), 256, s, c->p.gamma, c->nif, a.ifc, c->gadm[c->cur]);
+      k_adm<<<blocks(c->nif, 256), 256, 0, s>>>(c->p.gamma, c->nif, a.ifc, c->gadm[c->cur]);
       c->launches++;
     }
     a.adm_in = c->gadm[c->cur];
@@ -455,19 +502,27 @@ int enqueue_step(grp_ctx* c, double t_end)
   }
   if (c->p.solver != GRP_SOLVER_DET) a.fixed = flux_fixed(a) ? 1 : 0;
   const bool euler = c->p.system == GRP_EULER_IDEAL;
-  const unsigned tc = spread(c->ncell, 256), lb = list_blocks(c->ncell);
+  const unsigned tc = spread(c->ncell, 256), lb = LIST_BLOCKS;
+  // short grids of few domains: the time steps with S_max, the repair and the
+  // books in one launch
+  const bool small = euler && c->ncell <= SMALL_CELLS && c->D <= SMALL_DOMAINS;
+  // small grids: FP64 solves what it would list in place (the second pass would
+  // add its own latency to the first one's)
+  if (c->ncell <= FIXED_MIN_EQ_BATCH && c->p.solver != GRP_SOLVER_DET && !a.fixed && a.ph.guess != 2) a.hard_cap = 0;
   if (euler) {
     if (c->ncell <= SPEED_SMALL) {
-      chain(k_speed, blocks(c->ncell, tc), tc, s, a);
+      k_speed<<<blocks(c->ncell, tc), tc, 0, s>>>(a, small ? 1 : 0);
       c->launches++;
     } else {
-      chain(k_speed32, speed_blocks(c->ncell), 256, s, a);
-      chain(k_speed64, blocks(c->ncell, 256), 256, s, a);
+      k_speed32<<<speed_blocks(c->ncell), 256, 0, s>>>(a);
+      k_speed64<<<blocks(c->ncell, 256), 256, 0, s>>>(a);
       c->launches += 2;
     }
   }
-  chain(k_dt, blocks(c->D, 128), 128, s, a);
-  c->launches++;
+  if (!small) {
+    k_dt<<<blocks(c->D, 128), 128, 0, s>>>(a);
+    c->launches++;
+  }
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (c->timing) {
     for (cudaEvent_t* e : {&e0, &e1}) {
@@ -481,7 +536,7 @@ int enqueue_step(grp_ctx* c, double t_end)
     c->launches += 3;
   } else {
     CK(c->p.source != GRP_SOURCE_NONE ? launch_flux_src(a, s) : launch_flux(a, s));
-    c->launches += flux_defers(a) || a.fixed ? 2 : 1;
+    c->launches += (flux_defers(a) || a.fixed ? 2 : 1);
   }
   if (c->timing) {
     CK(record(c, e1));
@@ -489,21 +544,31 @@ int enqueue_step(grp_ctx* c, double t_end)
     c->ev_pending.push_back(e1);
   }
   if (euler) {
-    chain(k_update<SYS_EULER>, blocks(c->ncell, tc), tc, s, a, -1);
+    const bool p32 = c->ncell > SPEED_SMALL;                // FP32 densities and pressures kept with S_max
+    if (p32) k_update<SYS_EULER, true><<<blocks(c->ncell, tc), tc, 0, s>>>(a, -1);
+    else k_update<SYS_EULER, false><<<blocks(c->ncell, tc), tc, 0, s>>>(a, -1);
     c->launches++;
     // repair rounds over the compacted lists of troubled cells and repaired interfaces
-    for (int r = 0; r < MAX_REPAIR; ++r) {
-      if (c->p.gamma == 1.4) chain(k_repair_list<true>, lb, LIST_THREADS, s, a, r);
-      else chain(k_repair_list<false>, lb, LIST_THREADS, s, a, r);
-      chain(k_update_list<SYS_EULER>, lb, LIST_THREADS, s, a, r);
+    if (small) {
+      if (c->p.gamma == 1.4) k_tail<true><<<TAIL_BLOCKS, LIST_THREADS, 0, s>>>(a);
+      else k_tail<false><<<TAIL_BLOCKS, LIST_THREADS, 0, s>>>(a);
+      c->launches++;
+    }
+    for (int r = 0; r < MAX_REPAIR && !small; ++r) {
+      if (c->p.gamma == 1.4) k_repair_list<true><<<lb, LIST_THREADS, 0, s>>>(a, r);
+      else k_repair_list<false><<<lb, LIST_THREADS, 0, s>>>(a, r);
+      if (p32) k_update_list<SYS_EULER, true><<<lb, LIST_THREADS, 0, s>>>(a, r);
+      else k_update_list<SYS_EULER, false><<<lb, LIST_THREADS, 0, s>>>(a, r);
       c->launches += 2;
     }
   } else {
-    chain(k_update<SYS_ADV>, blocks(c->ncell, tc), tc, s, a, -1);
+    k_update<SYS_ADV, false><<<blocks(c->ncell, tc), tc, 0, s>>>(a, -1);
     c->launches++;
   }
-  chain(k_finish, blocks(c->D, 128), 128, s, a);
-  c->launches++;
+  if (!small) {
+    k_finish<<<blocks(c->D, 128), 128, 0, s>>>(a);
+    c->launches++;
+  }
   CK(cudaGetLastError());
   c->adm_valid = flags;
   c->cur ^= 1;
@@ -612,10 +677,10 @@ int grp_create(grp_ctx** out, const grp_problem* p)
   }
   AL(cell_off, D + 1) AL(if_off, D + 1) AL(cell_dom, c->ncell) AL(if_dom, c->nif) AL(dx, D) AL(bc, D)
   AL(avg[0], C * c->ncell) AL(avg[1], C * c->ncell) AL(ifc[0], C * c->nif) AL(ifc[1], C * c->nif)
-  AL(flux, C * c->nif) AL(pold, c->ncell) AL(slow32, D) AL(ds, D) AL(low, c->nif) AL(troubled, c->ncell) AL(t, D) AL(dt_prev, D) AL(nstep, D)
+  AL(flux, C * c->nif) AL(pold, c->ncell) AL(slow32, D) AL(ds, 2 * D) AL(low, c->nif) AL(troubled, c->ncell) AL(t, D) AL(dt_prev, D) AL(nstep, D)
   AL(status, D) AL(smax_bits, D) AL(bad, (MAX_REPAIR + 1) * D) AL(inad, D) AL(fail, D)
   AL(any_bad, MAX_REPAIR + 1) AL(stats, (long long)NSTATS * D) AL(scratch_norm, 3 * D)
-  AL(tlist0, c->ncell) AL(tlist1, c->ncell) AL(ilist, c->nif) AL(lcount, 2 * (MAX_REPAIR + 1))
+  AL(tlist0, c->ncell) AL(tlist1, c->ncell) AL(ilist, c->nif) AL(lcount, LCOUNT)
   if (p->source != GRP_SOURCE_NONE) AL(srcv, (long long)C * c->ncell)
   if (p->system == GRP_EULER_IDEAL && p->solver != GRP_SOLVER_DET && p->source == GRP_SOURCE_NONE) {
     c->hard_cap = c->nif;
@@ -680,21 +745,12 @@ int grp_set_initial(grp_ctx* c, const double* averages, const double* lim_minus,
     c->launches++;
     CK(cudaGetLastError());
   }
-  const int D = c->D;
-  CK(cudaMemsetAsync(c->t, 0, sizeof(double) * D, s));
-  CK(cudaMemsetAsync(c->dt_prev, 0, sizeof(double) * D, s));
-  CK(cudaMemsetAsync(c->nstep, 0, sizeof(int) * D, s));
-  CK(cudaMemsetAsync(c->status, 0, sizeof(int) * D, s));
-  CK(cudaMemsetAsync(c->smax_bits, 0, sizeof(unsigned long long) * D, s));
-  CK(cudaMemsetAsync(c->slow32, 0, sizeof(unsigned) * D, s));
-  CK(cudaMemsetAsync(c->stats, 0, sizeof(unsigned long long) * NSTATS * D, s));
-  CK(cudaMemsetAsync(c->low, 0, c->nif, s));
-  CK(cudaMemsetAsync(c->troubled, 0, c->ncell, s));
-  // per-domain repair and failure words: the flat form clears them every
-  // step, the block-local forms at the start of their first step
-  CK(cudaMemsetAsync(c->bad, 0, sizeof(int) * (MAX_REPAIR + 1) * D, s));
-  CK(cudaMemsetAsync(c->inad, 0, sizeof(int) * D, s));
-  CK(cudaMemsetAsync(c->fail, 0, sizeof(int) * D, s));
+  const StepArgs a = make_args(c, INFINITY);
+  const long long n = c->ncell > c->nif ? c->ncell : c->nif;
+  k_reset<<<blocks(n > c->D ? n : c->D, 256), 256, 0, s>>>(a);
+  c->launches++;
+  CK(cudaGetLastError());
+  c->ds_ready = false;
   c->initialized = true;
   c->host_steps = 0;
   c->smax_ready = false;
@@ -790,13 +846,6 @@ int enqueue_unit(grp_ctx* c, int k, double t_end)
   return GRP_OK;
 }
 
-unsigned long long bits_of(double x)
-{
-  unsigned long long b;
-  memcpy(&b, &x, sizeof b);
-  return b;
-}
-
 // Captures `steps` steps (whole launch units) starting from the context's
 // current buffer parity into a CUDA graph.  The kernels' arguments (buffer
 // pointers, t_end) are fixed in the graph, so a graph serves one start parity,
@@ -824,6 +873,9 @@ int capture_graph(grp_ctx* c, int steps, double t_end, grp_ctx::Graph& out)
   out.start_cur = c->cur;
   out.smax_ready = c->smax_ready;
   out.adm_valid = c->adm_valid;
+  const bool ds0 = c->ds_ready;
+  const unsigned long long dst0 = c->ds_t_end;
+  out.ds_ready = ds0 && dst0 == bits_of(t_end);
   out.t_end_bits = bits_of(t_end);
   out.steps = steps;
   const int cur0 = c->cur;
@@ -846,6 +898,9 @@ int capture_graph(grp_ctx* c, int steps, double t_end, grp_ctx::Graph& out)
   out.launches = c->launches - launches0;
   out.adm_end = c->adm_valid;
   c->adm_valid = adm0;
+  out.ds_end = c->ds_ready;
+  c->ds_ready = ds0;
+  c->ds_t_end = dst0;
   out.cur_end = c->cur;
   c->host_steps = hs0;
   // the timing events recorded during capture become nodes of the graph
@@ -888,7 +943,7 @@ int replay_graph(grp_ctx* c, double t_end)
   grp_ctx::Graph* G = nullptr;
   for (auto& g : c->graphs)
     if (g.start_cur == c->cur && g.smax_ready == c->smax_ready && g.adm_valid == c->adm_valid &&
-        g.t_end_bits == tb && g.steps == c->graph_steps)
+        g.ds_ready == (c->ds_ready && c->ds_t_end == tb) && g.t_end_bits == tb && g.steps == c->graph_steps)
       G = &g;
   if (!G) {
     if (c->graphs.size() >= 8) drop_graphs(c);      // t_end changed repeatedly: start over
@@ -911,6 +966,8 @@ int replay_graph(grp_ctx* c, double t_end)
   c->launches += G->launches;
   c->cur = G->cur_end;
   c->adm_valid = G->adm_end;
+  c->ds_ready = G->ds_end;
+  c->ds_t_end = tb;
   c->host_steps += G->steps;
   if (launch_form(c) == GRP_LAUNCH_SPLIT) c->smax_ready = true;
   else c->smax_ready = false;

@@ -232,7 +232,6 @@ __device__ __forceinline__ void det_finish(const StepArgs& a, const DetTab& T, l
 template <int SYS, int M, bool NL>
 __global__ void __launch_bounds__(128) k_det_predict(StepArgs a, double* __restrict__ ed, DetResume r)
 {
-  chain_wait();
   constexpr int n = M + 1, C = SYS == SYS_EULER ? 3 : 1;
   const long long gi = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (gi >= a.ncell) return;
@@ -291,7 +290,6 @@ __global__ void __launch_bounds__(128) k_det_predict(StepArgs a, double* __restr
 template <int SYS, int M>
 __global__ void __launch_bounds__(128) k_det_resume(StepArgs a, double* __restrict__ ed, DetResume r)
 {
-  chain_wait();
   constexpr int n = M + 1, C = SYS == SYS_EULER ? 3 : 1;
   const int cnt = *r.count < r.cap ? *r.count : r.cap;
   const DetTab& T = c_det[M - 1];
@@ -322,7 +320,6 @@ __global__ void __launch_bounds__(128) k_det_resume(StepArgs a, double* __restri
 template <int SYS, int M, bool G75>
 __global__ void __launch_bounds__(128) k_det_flux(StepArgs a, const double* __restrict__ ed)
 {
-  chain_wait();
   constexpr int n = M + 1, C = SYS == SYS_EULER ? 3 : 1;
   const long long gj = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   unsigned st[5] = {0u, 0u, 0u, 0u, 0u};   // newton sum, newton max, RS calls, first order
@@ -421,11 +418,11 @@ cudaError_t predict_launch(const StepArgs& a, double* ed, cudaStream_t s)
   const DetResume r = det_resume(M, C, a.ncell, ed);
   cudaError_t e = cudaMemsetAsync(r.count, 0, sizeof(int), s);
   if (e != cudaSuccess) return e;
-  chain(k_det_predict<SYS, M, NL>, (unsigned)((a.ncell + 127) / 128), 128, s, a, ed, r);
+  k_det_predict<SYS, M, NL><<<(unsigned)((a.ncell + 127) / 128), 128, 0, s>>>(a, ed, r);
   // one thread per slot of the list (its capacity fixes the grid, so a
   // captured graph serves every step; blocks past the count exit at once):
   // the listed cells iterate side by side, not one after another
-  chain(k_det_resume<SYS, M>, (unsigned)((r.cap + 127) / 128), 128, s, a, ed, r);
+  k_det_resume<SYS, M><<<(unsigned)((r.cap + 127) / 128), 128, 0, s>>>(a, ed, r);
   return cudaGetLastError();
 }
 
@@ -433,8 +430,8 @@ template <int SYS, int M>
 cudaError_t flux_launch(const StepArgs& a, const double* ed, cudaStream_t s)
 {
   const unsigned g = (unsigned)((a.nif + 127) / 128);
-  if (SYS == SYS_EULER && a.ph.gamma == 1.4) chain(k_det_flux<SYS, M, true>, g, 128, s, a, ed);
-  else chain(k_det_flux<SYS, M, false>, g, 128, s, a, ed);
+  if (SYS == SYS_EULER && a.ph.gamma == 1.4) k_det_flux<SYS, M, true><<<g, 128, 0, s>>>(a, ed);
+  else k_det_flux<SYS, M, false><<<g, 128, 0, s>>>(a, ed);
   return cudaGetLastError();
 }
 

@@ -501,9 +501,11 @@ GRP_HD __forceinline__ void riemann(const Consts& K, State& L, State& R, State& 
   d = add(d, (fx)(fabsf(s1) < 0x1p-16f ? s1 * 0x1p61f : 0.0f));
   const fx pl = pressure(L, c2[0], iL, d, G), pr = pressure(R, c2[1], iR, sub(du, d), G);
   const float s2 = to_f32(sub(pl, pr)) * inv;
-  const fx step = (fx)(fabsf(s2) < 0x1p-16f ? s2 * 0x1p61f : 0.0f);
-  const fx ps = sub(pl, (fx)(s2 * kl * (fabsf(s2) < 0x1p-16f ? 0x1p61f : 0.0f)));
-  d = add(d, step);
+  // the last step along the tangents; p* from both sides alike (a mirrored problem
+  // gives the mirrored state)
+  const float t2 = fabsf(s2) < 0x1p-16f ? s2 : 0.0f;
+  const fx ps = add(add(pl >> 1, pr >> 1), (fx)(0.5f * (kr - kl) * t2 * 0x1p61f));
+  d = add(d, (fx)(t2 * 0x1p61f));
   const fx us = add(L.u, d);
   // ---- the state at x / t = 0: the side of the contact, mirrored to the left
   const fx cc = add(L.c, R.c);

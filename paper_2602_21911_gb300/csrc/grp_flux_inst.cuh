@@ -13,8 +13,10 @@ inline bool launch_flux_fixed(const StepArgs& a, cudaStream_t s)
 {
   if (!a.fixed) return false;
   const unsigned tpb = spread(a.nif, 128);
-  if constexpr (!NLV) chain(k_flux_fixed<MM>, (unsigned)((a.nif + tpb - 1) / tpb), tpb, s, a);
-  else if constexpr (MM <= 3) chain(k_flux_fixed_nl<MM>, (unsigned)((flux_threads(a.nif) + tpb - 1) / tpb), tpb, s, a);
+  if constexpr (!NLV) {
+    k_flux_fixed<MM><<<(unsigned)((a.nif + tpb - 1) / tpb), tpb, 0, s>>>(a);
+  }
+  else if constexpr (MM <= 3) k_flux_fixed_nl<MM><<<(unsigned)((flux_threads(a.nif) + tpb - 1) / tpb), tpb, 0, s>>>(a);
   return true;
 }
 
@@ -34,14 +36,14 @@ inline void launch_flux_hard(const StepArgs& a, cudaStream_t s)
       if constexpr (DEFER) {
         const bool net = flux_hard_net(a);
         if (a.ph.gamma == 1.4) {
-          if (net) chain(k_flux_hard<MM, true, true>, gh, GRP_HARD_TPB, s, a);
-          else chain(k_flux_hard<MM, true, false>, gh, GRP_HARD_TPB, s, a);
+          if (net) k_flux_hard<MM, true, true><<<gh, GRP_HARD_TPB, 0, s>>>(a);
+          else k_flux_hard<MM, true, false><<<gh, GRP_HARD_TPB, 0, s>>>(a);
         } else {
-          if (net) chain(k_flux_hard<MM, false, true>, gh, GRP_HARD_TPB, s, a);
-          else chain(k_flux_hard<MM, false, false>, gh, GRP_HARD_TPB, s, a);
+          if (net) k_flux_hard<MM, false, true><<<gh, GRP_HARD_TPB, 0, s>>>(a);
+          else k_flux_hard<MM, false, false><<<gh, GRP_HARD_TPB, 0, s>>>(a);
         }
       } else {
-        chain(k_flux_hard<MM, true, false, NLV>, gh, GRP_HARD_TPB, s, a);      // gamma = 7/5 only
+        k_flux_hard<MM, true, false, NLV><<<gh, GRP_HARD_TPB, 0, s>>>(a);      // gamma = 7/5 only
       }
     }
   }
@@ -53,8 +55,8 @@ inline void launch_flux_hard(const StepArgs& a, cudaStream_t s)
   {                                                                                                          \
     const unsigned tpb = spread(a.nif, GRP_FLUX_TPB), g = (unsigned)((flux_threads(a.nif) + tpb - 1) / tpb); \
     if (launch_flux_fixed<MM, NLV>(a, s)) {}                                                                 \
-    else if (a.ph.gamma == 1.4) chain(k_flux<SYS_EULER, MM, true, NLV>, g, tpb, s, a);              \
-    else chain(k_flux<SYS_EULER, MM, false, NLV>, g, tpb, s, a);                                    \
+    else if (a.ph.gamma == 1.4) k_flux<SYS_EULER, MM, true, NLV><<<g, tpb, 0, s>>>(a);              \
+    else k_flux<SYS_EULER, MM, false, NLV><<<g, tpb, 0, s>>>(a);                                    \
     launch_flux_hard<MM, NLV>(a, s);                                                                         \
     return cudaGetLastError();                                                                               \
   }                                                                                                          \
@@ -74,10 +76,22 @@ inline void launch_flux_hard(const StepArgs& a, cudaStream_t s)
   {                                                                                                          \
     const unsigned tpb = spread(a.nif, GRP_FLUX_TPB), g = (unsigned)((flux_threads(a.nif) + tpb - 1) / tpb); \
     switch (a.M) {                                                                                           \
-      case 1: chain(k_flux<SYS_ADV, 1, false, NLV>, g, tpb, s, a); break;                                    \
-      case 2: chain(k_flux<SYS_ADV, 2, false, NLV>, g, tpb, s, a); break;                                    \
-      case 3: chain(k_flux<SYS_ADV, 3, false, NLV>, g, tpb, s, a); break;                                    \
-      case 4: chain(k_flux<SYS_ADV, 4, false, NLV>, g, tpb, s, a); break;                                    \
+      case 1: k_flux<SYS_ADV, 1, false, NLV><<<g, tpb, 0, s>>>(a); break;                                    \
+      case 2: k_flux<SYS_ADV, 2, false, NLV><<<g, tpb, 0, s>>>(a); break;                                    \
+      case 3: k_flux<SYS_ADV, 3, false, NLV><<<g, tpb, 0, s>>>(a); break;                                    \
+      case 4: k_flux<SYS_ADV, 4, false, NLV><<<g, tpb, 0, s>>>(a); break;                                    \
+      default: return cudaErrorInvalidValue;                                                                 \
+    }                                                                                                        \
+    return cudaGetLastError();                                                                               \
+  }                                                                                                          \
+  cudaError_t launch_adv_step##SUFFIX(const StepArgs& a, DomStep* next, cudaStream_t s)                      \
+  {                                                                                                          \
+    const unsigned tpb = spread(a.ncell, 256), g = (unsigned)((a.ncell + tpb - 1) / tpb);                    \
+    switch (a.M) {                                                                                           \
+      case 1: k_adv_step<1, NLV><<<g, tpb, 0, s>>>(a, next); break;                                          \
+      case 2: k_adv_step<2, NLV><<<g, tpb, 0, s>>>(a, next); break;                                          \
+      case 3: k_adv_step<3, NLV><<<g, tpb, 0, s>>>(a, next); break;                                          \
+      case 4: k_adv_step<4, NLV><<<g, tpb, 0, s>>>(a, next); break;                                          \
       default: return cudaErrorInvalidValue;                                                                 \
     }                                                                                                        \
     return cudaGetLastError();                                                                               \

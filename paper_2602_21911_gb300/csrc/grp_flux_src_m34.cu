@@ -10,12 +10,12 @@ cudaError_t launch_flux_src_m34(const StepArgs& a, cudaStream_t s)
   const bool g75 = a.ph.gamma == 1.4;
   switch (a.M) {
     case 3:
-      if (g75) chain(k_flux<SYS_EULER, 3, true, false, true>, g, tpb, s, a);
-      else chain(k_flux<SYS_EULER, 3, false, false, true>, g, tpb, s, a);
+      if (g75) k_flux<SYS_EULER, 3, true, false, true><<<g, tpb, 0, s>>>(a);
+      else k_flux<SYS_EULER, 3, false, false, true><<<g, tpb, 0, s>>>(a);
       break;
     case 4:
-      if (g75) chain(k_flux<SYS_EULER, 4, true, false, true>, g, tpb, s, a);
-      else chain(k_flux<SYS_EULER, 4, false, false, true>, g, tpb, s, a);
+      if (g75) k_flux<SYS_EULER, 4, true, false, true><<<g, tpb, 0, s>>>(a);
+      else k_flux<SYS_EULER, 4, false, false, true><<<g, tpb, 0, s>>>(a);
       break;
     default: return cudaErrorInvalidValue;
   }

@@ -1,20 +1,26 @@
 // Kernels of one FV+GRPrec time step over a flat batch of 1D domains.
 //
-// One step is a short fixed sequence of launches on the context's stream:
+// One step of the Euler equations is a short fixed sequence of launches on the
+// context's stream:
 //   k_speed32      per cell   FP32 bounds of |u| + c, density and pressure in FP32
 //   k_speed64      per cell   S_max of every domain from the cells that can hold it
-//   k_flux<M>      per iface  GRPrec traces -> GRP -> flux, new interface data
+//                  (k_speed does both for all but large grids)
+//   k_dt           per domain the time step
+//   k_flux_fixed   per iface  GRPrec traces -> GRP -> flux, new interface data, in
+//                  64-bit fixed point (k_flux: the same in FP64, see flux_fixed)
+//   k_flux_hard    per listed interface: what the pass before left, in FP64
 //   k_update       per cell   candidate averages, detection flags, list of troubled cells
 //   k_repair_list  per listed troubled cell: first-order fluxes on its interfaces
 //   k_update_list  per listed repaired interface: candidates of its cells again
 //                  (the last two MAX_REPAIR times, on fixed grids)
 //   k_finish       per domain time, step count, status, buffer bookkeeping
+// On short grids of few domains k_speed forms the time steps too and k_tail does all
+// repair rounds and the bookkeeping.  Advection takes one launch, k_adv_step.
 // Every kernel derives dt from the same per-domain words with the same
 // expression, so no extra launch is needed to publish it.
 #pragma once
 #include "grp_device.cuh"
 #include "grp_fixed.cuh"
-#include "grp_launch.h"
 
 namespace grp {
 
@@ -22,6 +28,9 @@ constexpr int NSTATS = 9;
 enum { S_STEPS = 0, S_NEWTON_SUM, S_NEWTON_MAX, S_RECON_FB, S_FLUX_FB, S_RS_CALLS, S_LOW, S_GUESS_USED,
        S_GUESS_REJ };
 constexpr int MAX_REPAIR = 4;   // rounds of the a-posteriori first-order repair
+constexpr long long SMALL_CELLS = 152 * 64;      // a short grid: two warps of cells per SM at most ...
+constexpr int SMALL_DOMAINS = 16;                // ... of few domains
+constexpr int LCOUNT = 2 * (MAX_REPAIR + 1) + 1;   // words of lcount
 constexpr double DMP_REL = 1e-2; // relaxation of the discrete maximum principle
 
 // This step's time step of one domain, computed once per step after S_max.
@@ -75,8 +84,8 @@ struct StepArgs {
   // troubled cells and their interfaces)
   int* tlist[2];                     // [ncell] troubled cells after pass p-1, in tlist[p & 1]
   int* ilist;                        // [nif] interfaces repaired in the current round
-  int* lcount;                       // [2 (MAX_REPAIR+1)]: troubled cells after pass p-1 at [p];
-                                     //   interfaces repaired in round r at [MAX_REPAIR + 1 + r]
+  int* lcount;                       // [LCOUNT]: troubled cells after pass p-1 at [p]; interfaces repaired in
+                                     //   round r at [MAX_REPAIR + 1 + r]; blocks done (k_speed), 0 between launches
   unsigned long long* stats;         // [D][NSTATS]
   // interfaces of the flux kernel deferred to k_flux_hard (Riemann data that
   // are not equal data, at the interpolating degrees; interfaces outside the
@@ -155,7 +164,7 @@ __device__ __forceinline__ void warp_flux_stats(unsigned long long* stats, int d
 // Time-step rule (Section 4.1): dt = C dx / S_max, recomputed every dt_hold
 // steps, the last step clipped to t_end.  false: the domain does not move.
 // Time step of domain d from its words (S_max complete): one division.
-__device__ __forceinline__ void compute_domain_step(const StepArgs& a, int d)
+__device__ __forceinline__ DomStep domain_step(const StepArgs& a, int d)
 {
   DomStep r{0.0, 0.0, 0.0, 0, 0, {0.0, 0.0, 0.0}};
   const double t = a.t[d];
@@ -163,7 +172,7 @@ __device__ __forceinline__ void compute_domain_step(const StepArgs& a, int d)
     const double dtp = a.dt_prev[d];
     double dt_cfl;
     if (a.nstep[d] % a.dt_hold == 0 || !(dtp > 0.0)) {
-      const double smax = a.sys == SYS_ADV ? fabs(a.ph.lambda) : __longlong_as_double((long long)a.smax_bits[d]);
+      const double smax = a.sys == SYS_ADV ? fabs(a.ph.lambda) : __longlong_as_double((long long)__ldcg(a.smax_bits + d));
       dt_cfl = __ddiv_rn(__dmul_rn(a.cfl, a.dx[d]), smax);
     } else {
       dt_cfl = dtp;
@@ -178,8 +187,9 @@ __device__ __forceinline__ void compute_domain_step(const StepArgs& a, int d)
     for (int al = 0; al < G; ++al) r.tg[al] = __dmul_rn(r.nu, gauss_node(G, al));
     r.active = 1;
   }
-  a.ds[d] = r;
+  return r;
 }
+__device__ __forceinline__ void compute_domain_step(const StepArgs& a, int d) { a.ds[d] = domain_step(a, d); }
 
 // The step's time step of domain d; false when the domain does not step.
 __device__ __forceinline__ bool domain_dt(const StepArgs& a, int d, double& dt, double& dt_cfl, bool& last)
@@ -194,18 +204,20 @@ __device__ __forceinline__ bool domain_dt(const StepArgs& a, int d, double& dt, 
 // Per-domain words of the step: repair flags and failure code cleared (every
 // system; the S_max pass clears them too for the Euler equations), then the
 // time step.
+__device__ __forceinline__ void begin_domain(const StepArgs& a, int d)
+{
+  for (int p = 0; p <= MAX_REPAIR; ++p) a.bad[p * a.n_domains + d] = 0;
+  a.inad[d] = 0;
+  a.fail[d] = 0;
+  const DomStep r = domain_step(a, d);
+  a.ds[d] = r;
+  if (a.fixed && r.active)
+    a.stats[(long long)d * NSTATS + S_RS_CALLS] += (unsigned long long)(a.if_off[d + 1] - a.if_off[d]);
+}
 static __global__ void k_dt(StepArgs a)
 {
-  chain_wait();
   const int d = blockIdx.x * blockDim.x + threadIdx.x;
-  if (d < a.n_domains) {
-    for (int p = 0; p <= MAX_REPAIR; ++p) a.bad[p * a.n_domains + d] = 0;
-    a.inad[d] = 0;
-    a.fail[d] = 0;
-    compute_domain_step(a, d);
-    if (a.fixed && a.ds[d].active)
-      a.stats[(long long)d * NSTATS + S_RS_CALLS] += (unsigned long long)(a.if_off[d + 1] - a.if_off[d]);
-  }
+  if (d < a.n_domains) begin_domain(a, d);
 }
 
 // Neighbour cells of cell i (domain-local) under the domain's boundary rule:
@@ -308,7 +320,6 @@ inline unsigned speed_blocks(long long ncell) { return (unsigned)((ncell + 256 *
 
 static __global__ void __launch_bounds__(256) k_speed32(StepArgs a)
 {
-  chain_wait();
   if (blockIdx.x == 0 && threadIdx.x <= MAX_REPAIR) a.any_bad[threadIdx.x] = 0;
   if (blockIdx.x == 0 && threadIdx.x < 2 * (MAX_REPAIR + 1)) a.lcount[threadIdx.x] = 0;
   const long long g0 = (long long)blockIdx.x * (256 * SPEED_CELLS) + threadIdx.x;
@@ -343,12 +354,16 @@ static __global__ void __launch_bounds__(256) k_speed32(StepArgs a)
   }
 }
 
-// Both in one FP64 launch, for grids that leave the GPU mostly idle (the two
-// passes' latencies add up there: 7 us on a domain of 200 cells).
-constexpr long long SPEED_SMALL = 1 << 17;
-static __global__ void __launch_bounds__(256) k_speed(StepArgs a)
+// Both in one FP64 launch, for smaller grids (the two passes' latencies add up
+// there: 7 us on a domain of 200 cells); the update then takes the FP64 test with
+// the pressures kept here (the FP32 test first is longer for each repair round).
+// Measured: at 6.9 M cells the FP32 forms take 194 us a step off, 2.8 us per
+// 100,000 cells; at 115,000 cells the step was 5 us longer with them; the line is
+// drawn above the 300,000 where the two meet.
+// turn: the last block to finish also takes the domains' time steps (k_dt's work).
+constexpr long long SPEED_SMALL = 400000;
+static __global__ void __launch_bounds__(256) k_speed(StepArgs a, int turn)
 {
-  chain_wait();
   if (blockIdx.x == 0 && threadIdx.x <= MAX_REPAIR) a.any_bad[threadIdx.x] = 0;
   if (blockIdx.x == 0 && threadIdx.x < 2 * (MAX_REPAIR + 1)) a.lcount[threadIdx.x] = 0;
   const long long gi = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -363,8 +378,7 @@ static __global__ void __launch_bounds__(256) k_speed(StepArgs a)
     const double sp = fabs(u) + (positive(c2) ? c2 * rsqrt(c2) : 0.0);
     const long long sb = __double_as_longlong(sp);
     if (sb >= 0ll && sb <= 0x7ff0000000000000ll) { hi = (unsigned)(sb >> 32); lo = (unsigned)sb; }
-    const float rf = trunc32(r), pf = trunc32(p), cap = a.gm1f * trunc32(E);
-    a.rp32[gi] = make_float2(rf, rf > 1e-30f && cap > 1e-30f && cap < 1e30f && pf > cap * 0x1p-9f ? pf : NAN);
+    a.pold[gi] = p;
   }
   // the largest 64-bit pattern of the warp's cells of one domain, in two words
   const unsigned grp = __match_any_sync(0xffffffffu, d);
@@ -372,13 +386,23 @@ static __global__ void __launch_bounds__(256) k_speed(StepArgs a)
   const unsigned ml = __reduce_max_sync(grp, hi == mh ? lo : 0u);
   if (d >= 0 && lane_id() == __ffs(grp) - 1)
     atomicMax(a.smax_bits + d, ((unsigned long long)mh << 32) | ml);
+  if (!turn) return;
+  __shared__ bool last;
+  __threadfence();
+  __syncthreads();
+  int* done = a.lcount + LCOUNT - 1;
+  if (threadIdx.x == 0) last = atomicAdd(done, 1) == (int)gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  for (int k = threadIdx.x; k < a.n_domains; k += blockDim.x) begin_domain(a, k);
+  if (threadIdx.x == 0) *done = 0;
 }
 
 // FP64 pass over the cells that can hold the maximum.  Runs of identical
 // states (undisturbed gas) are evaluated at their first cell.
 static __global__ void __launch_bounds__(256) k_speed64(StepArgs a)
 {
-  chain_wait();
   const long long gi = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (gi >= a.ncell) return;
   const int d = a.cell_dom[gi];
@@ -887,7 +911,6 @@ __device__ __forceinline__ void count_newton(const StepArgs& a, bool newton, int
 template <int M>
 __global__ void __launch_bounds__(128, M == 2 ? 5 : 3) k_flux_fixed(StepArgs a)
 {
-  chain_wait();
   constexpr bool EQ = M == 2 || M == 4;
   constexpr int NQ = M <= 2 ? 2 : 4, IL = M <= 2 ? 0 : 1;
   const long long gj = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -952,7 +975,6 @@ __global__ void __launch_bounds__(128, M == 2 ? 5 : 3) k_flux_fixed(StepArgs a)
 template <int M>
 __global__ void __launch_bounds__(128, 3) k_flux_fixed_nl(StepArgs a)
 {
-  chain_wait();
   const int lane = lane_id();
   const long long gj = (((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 31 + lane;
   bool hard = false, newton = false, active = false, fb = false;
@@ -1016,7 +1038,6 @@ __host__ __device__ constexpr bool flux_defers_at()
 template <int SYS, int M, bool G75, bool NL, bool SRC = false>
 __global__ void __launch_bounds__(GRP_FLUX_TPB, GRP_FLUX_MIN_BLOCKS) k_flux(StepArgs a)
 {
-  chain_wait();
   flux_warp<SYS, M, G75, NL, SRC, flux_defers_at<SYS, M, NL, SRC>()>(
       a, (((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 31, a.nif);
 }
@@ -1033,15 +1054,32 @@ inline bool flux_defers(const StepArgs& a)
 // The Riemann problems of the other degrees and of GRPrecNL are solved for
 // gamma = 7/5 and to the format's precision whatever newton_rtol asks beyond it;
 // the learned start and the harvest keep the FP64 pass, whose iterations they
-// are about.  Degree 4 on less than two warps per SM stays in FP64: one warp
-// alone takes 38 us in fixed point and 26 us in FP64 (degree 2: 10 and 14 us).
-constexpr long long FIXED_MIN4 = 152 * 64;
+// are about.
+// Smaller grids with open ends stay in FP64: their step is a chain of latencies,
+// and the second pass (the ends at least) adds its own to the first one's, where
+// FP64 solves everything in place.  Measured, us per step, fixed point / FP64 in
+// place: tube of 12,000 cells 58 / 51 (degree 2) and 76 / 64 (degree 4), of 20,000
+// 58 / 57 and 79 / 81, of 40,000 63 / 67 and 88 / 101; 2,330 domains of 22 cells
+// 195 / 186 and 239 / 221; domains of 38 cells, 1,400 of them
+// 185 / 174 and 235 / 227, 2,000 of them 205 / 202 and 257 / 266.  The Riemann
+// problems of degrees 1 and 3: 300 domains of 38 cells at degree 3 164 / 144.
+// Periodic grids have no ends: wave of 9,000 cells 23 / 27, degree 3 32 / 53.
+constexpr long long FIXED_MIN_EQ = 152 * 128, FIXED_MIN_EQ_BATCH = 72000, FIXED_MIN_RP = 152 * 192,
+                    FIXED_MIN_RP_BATCH = 192000, FIXED_MIN_NL = 400000;
+inline bool fixed_riemann(const StepArgs& a)
+{
+  return a.ph.gamma == 1.4 && a.ph.guess != 2 && !a.harvest && a.ph.rtol >= 1e-13 && a.ph.max_iter >= (int)FIXED_ITERS;
+}
 inline bool flux_fixed(const StepArgs& a)
 {
   if (a.sys != SYS_EULER || a.srcv || a.hard_cap == 0 || !fixed::gamma_ok(a.ph.gamma)) return false;
-  if (a.recon == 0 && (a.M == 2 || a.M == 4)) return a.adm_in && (a.M == 2 || a.nif > FIXED_MIN4);
-  return a.ph.gamma == 1.4 && (a.recon == 0 || a.M <= 3) && a.ph.guess != 2 && !a.harvest && a.ph.rtol >= 1e-13 &&
-         a.ph.max_iter >= (int)FIXED_ITERS;
+  const bool eq = a.recon == 0 && (a.M == 2 || a.M == 4);
+  const bool few = a.n_domains <= SMALL_DOMAINS;
+  const long long least = eq ? (few ? FIXED_MIN_EQ : FIXED_MIN_EQ_BATCH)
+                             : few ? FIXED_MIN_RP : a.recon ? FIXED_MIN_NL : FIXED_MIN_RP_BATCH;
+  if (a.nif != a.ncell && a.nif <= least) return false;                // (nif = ncell: no open end)
+  if (eq) return a.adm_in != nullptr;
+  return (a.recon == 0 || a.M <= 3) && fixed_riemann(a);
 }
 
 // The second pass runs one warp per block, so that a warp that finishes frees
@@ -1061,6 +1099,8 @@ inline unsigned hard_blocks(long long cap, int sms)
   return (unsigned)(need < fill ? need : fill);
 }
 
+constexpr long long HARD_HALF = 16 * 1216;   // a list of at most 16 interfaces a warp at eight warps per SM
+
 // The second pass of the flux kernel: the deferred interfaces, one per lane
 // (a warp takes its chunk together, so the warp statistics see full warps).
 // The last block to finish resets the list for the next step; every block
@@ -1071,23 +1111,32 @@ inline unsigned hard_blocks(long long cap, int sms)
 template <int M, bool G75, bool NET, bool NL = false>
 __global__ void __launch_bounds__(GRP_HARD_TPB, GRP_HARD_MIN_BLOCKS) k_flux_hard(StepArgs a)
 {
-  chain_wait();
   constexpr int C = 3;
   const unsigned offered = a.hard_count[0];
   const long long n = offered < (unsigned)a.hard_cap ? offered : a.hard_cap;
   const int lane = lane_id();
   __shared__ float hs[NET ? GRP_HARD_TPB / 32 : 1][MLP_NH];
+  // A short list is spread over eight warps per SM, a few interfaces each: the
+  // fewer lanes, the fewer branches of the solver a warp takes in turn (86,000
+  // cells, us per step: 230 with eight warps, 234 with four, 242 with full warps).
+  // With 16 or fewer interfaces the upper half of the warp forms the right cells' traces
+  // while the lower half forms the left cells'.
+  const unsigned spread_n = (unsigned)((n + 1215) / 1216);
+  const bool half = n <= HARD_HALF;
+  const unsigned most = half ? 16u : 32u, chunk = spread_n < most ? (spread_n > 0u ? spread_n : 1u) : most;
+  const unsigned slot = half ? lane & 15u : lane;
+  const bool right = half && lane >= 16;
   for (;;) {
     unsigned b = 0;
-    if (lane == 0) b = atomicAdd(a.hard_count + 2, 32u);
+    if (lane == 0) b = atomicAdd(a.hard_count + 2, chunk);
     b = __shfl_sync(0xffffffffu, b, 0);
     if ((long long)b >= n) break;
-    const long long i = (long long)b + lane;
+    const long long i = (long long)b + slot;
     unsigned st[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
     int d = -1;
     long long gj = 0;
-    double tL[C][M + 1], tR[C][M + 1];
-    if (i < n) {
+    double tL[C][M + 1], tR[C][M + 1], em[C][M + 1], ep[C][M + 1];
+    if (i < n && slot < chunk) {
       gj = a.hard_idx[i];
       d = a.if_dom[gj];
       // the traces again: both cells' reconstructions, or the ghost state
@@ -1095,13 +1144,29 @@ __global__ void __launch_bounds__(GRP_HARD_TPB, GRP_HARD_MIN_BLOCKS) k_flux_hard
       const int N = (int)(a.cell_off[d + 1] - c0), bc = a.bc[d], j = (int)(gj - i0);
       const int cl = bc == 0 ? (j == 0 ? N - 1 : j - 1) : j - 1, cr = bc != 0 && j == N ? -1 : j;
       constexpr bool EQ = !NL && (M == 2 || M == 4);
-      double tx[C][M + 1];
-      bool fb = false;
-      if (cl >= 0) cell_edges<SYS_EULER, M, NL, EQ>(a, c0, i0, N, bc, cl, tx, tL, fb);
-      else ghost_edge<SYS_EULER, M>(a, c0, 0, tL);
-      if (!EQ) st[5] = fb ? 1u : 0u;               // (degrees 2 and 4: counted by the first pass, from the flags)
-      if (cr >= 0) cell_edges<SYS_EULER, M, NL, EQ>(a, c0, i0, N, bc, cr, tR, tx, fb);
-      else ghost_edge<SYS_EULER, M>(a, c0, N - 1, tR);
+      // (not unrolled: one copy of the reconstruction's code)
+#pragma unroll 1
+      for (int k = right ? 1 : 0; k < (half && !right ? 1 : 2); ++k) {
+        const int cell = k ? cr : cl;
+        bool fb = false;
+        if (cell >= 0) cell_edges<SYS_EULER, M, NL, EQ>(a, c0, i0, N, bc, cell, em, ep, fb);
+        else ghost_edge<SYS_EULER, M>(a, c0, k ? N - 1 : 0, em);
+#pragma unroll
+        for (int c = 0; c < C; ++c)
+#pragma unroll
+          for (int m = 0; m <= M; ++m) {
+            if (k) tR[c][m] = em[c][m];
+            else tL[c][m] = cell >= 0 ? ep[c][m] : em[c][m];
+          }
+        if (!EQ && k == 0) st[5] = fb ? 1u : 0u;   // (degrees 2 and 4: counted by the first pass, from the flags)
+      }
+    }
+    if (half) {
+#pragma unroll
+      for (int c = 0; c < C; ++c)
+#pragma unroll
+        for (int k = 0; k <= M; ++k) tR[c][k] = __shfl_down_sync(0xffffffffu, tR[c][k], 16);
+      if (right) d = -1;
     }
     if (NET) {
       Side L, R;
@@ -1233,13 +1298,14 @@ __device__ __forceinline__ int update_one(const StepArgs& a, long long gi, int d
     a.avg_new[c * a.ncell + gi] = Q[c];
   }
   if (SYS != SYS_EULER) return 0;
-  if (P32 && pass < 0) {
+  if (P32) {
     int im, ip;
     nbr(i, N, a.bc[d], im, ip);
     const int f = dmp32(a, a.rp32[c0 + im], a.rp32[gi], a.rp32[c0 + ip], Q);
     if (f >= 0) {
+      if (pass >= 0 && a.troubled[gi] == 2) atomicSub(a.inad + d, 1);
       a.troubled[gi] = (unsigned char)f;
-      if (f) a.bad[d] = 1;
+      if (f) a.bad[(pass + 1) * a.n_domains + d] = 1;
       return f;
     }
   }
@@ -1290,15 +1356,14 @@ __device__ __forceinline__ int update_one(const StepArgs& a, long long gi, int d
   return (ok ? 0 : 1) | (adm ? 0 : 2);
 }
 
-template <int SYS>
-__global__ void __launch_bounds__(256, 8) k_update(StepArgs a, int pass)
+template <int SYS, bool P32>
+__global__ void __launch_bounds__(256, P32 ? 8 : 1) k_update(StepArgs a, int pass)
 {
-  chain_wait();
   const long long gi = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (pass >= 0 && a.any_bad[pass] == 0) return;
   if (gi >= a.ncell) return;
   const int d = a.cell_dom[gi];
-  const bool bad = update_one<SYS, SYS == SYS_EULER>(a, gi, d, pass) & 1;
+  const bool bad = update_one<SYS, P32>(a, gi, d, pass) & 1;
   if (bad) a.any_bad[pass + 1] = 1;
   if (pass < 0 && a.lcount) {
     // warp-aggregated append of the troubled cells to the first work list
@@ -1317,8 +1382,11 @@ __global__ void __launch_bounds__(256, 8) k_update(StepArgs a, int pass)
 // Grid-stride helpers of the work-list kernels (their grids are fixed, so a
 // captured graph serves every step).
 constexpr int LIST_BLOCKS = 4 * 152, LIST_THREADS = 128;
-inline unsigned list_blocks(long long) { return LIST_BLOCKS; }
-inline unsigned spread(long long n, unsigned threads) { (void)n; return threads; }
+// Threads per block of a kernel over n cells or interfaces: small grids are cut
+// into one-warp blocks, which spread over the SMs (the FP64 unit of an SM serves
+// one warp instruction in 16 cycles, so warps on SMs of their own run side by
+// side).
+inline unsigned spread(long long n, unsigned threads) { return n <= 152 * 64 ? 32u : threads; }
 
 // First-order Godunov flux at interface gj (round `pass`); appends it to the
 // round's interface list.
@@ -1358,12 +1426,11 @@ __device__ __forceinline__ void repair_iface(const StepArgs& a, int pass, long l
 // gathers the named interfaces of its slice of the list in shared memory and
 // then solves them one per thread, so the warps running Riemann problems are
 // full (on this GPU a divergent FP64 instruction costs as much as a full one).
+// q: 2 blockDim words and qn of shared memory; the calling grid's blocks share the
+// list.
 template <bool G75>
-__global__ void __launch_bounds__(LIST_THREADS) k_repair_list(StepArgs a, int pass)
+__device__ __forceinline__ void repair_round(const StepArgs& a, int pass, long long* q, int& qn)
 {
-  chain_wait();
-  __shared__ long long q[2 * LIST_THREADS];
-  __shared__ int qn;
   const int n = a.lcount[pass];
   const int* L = a.tlist[pass & 1];
   // the list spread evenly over the whole grid: a short list gives every
@@ -1393,15 +1460,22 @@ __global__ void __launch_bounds__(LIST_THREADS) k_repair_list(StepArgs a, int pa
   }
 }
 
+template <bool G75>
+__global__ void __launch_bounds__(LIST_THREADS) k_repair_list(StepArgs a, int pass)
+{
+  __shared__ long long q[2 * LIST_THREADS];
+  __shared__ int qn;
+  repair_round<G75>(a, pass, q, qn);
+}
+
 // Re-update after round `pass` from the list of repaired interfaces.  The
 // cells next to interface j are its right cell (whose left interface is j)
 // and its left cell; the left cell is left to its own left interface when
 // that was repaired in this round too, so every cell is updated once.
 // Troubled results go to the next round's cell list.
-template <int SYS>
-__global__ void __launch_bounds__(LIST_THREADS) k_update_list(StepArgs a, int pass)
+template <int SYS, bool P32>
+__device__ __forceinline__ void update_round(const StepArgs& a, int pass)
 {
-  chain_wait();
   const int n = a.lcount[MAX_REPAIR + 1 + pass];
   const unsigned char mark = (unsigned char)(2 + pass);
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
@@ -1419,12 +1493,18 @@ __global__ void __launch_bounds__(LIST_THREADS) k_update_list(StepArgs a, int pa
     if (cl >= 0 && a.low[i0 + cl] != mark) cells[nc++] = cl;
     for (int q = 0; q < nc; ++q) {
       const long long gi = c0 + cells[q];
-      if (update_one<SYS, SYS == SYS_EULER>(a, gi, d, pass) & 1) {
+      if (update_one<SYS, P32>(a, gi, d, pass) & 1) {
         a.any_bad[pass + 1] = 1;
         if (pass + 1 <= MAX_REPAIR) a.tlist[(pass + 1) & 1][atomicAdd(a.lcount + pass + 1, 1)] = (int)gi;
       }
     }
   }
+}
+
+template <int SYS, bool P32>
+__global__ void __launch_bounds__(LIST_THREADS) k_update_list(StepArgs a, int pass)
+{
+  update_round<SYS, P32>(a, pass);
 }
 
 // ------------------------------------------------------------------ repair
@@ -1482,9 +1562,94 @@ __device__ __forceinline__ void finish_one(const StepArgs& a, int d)
 
 static __global__ void k_finish(StepArgs a)
 {
-  chain_wait();
   const int d = blockIdx.x * blockDim.x + threadIdx.x;
   if (d < a.n_domains) finish_one(a, d);
+}
+
+// All repair rounds and the bookkeeping of a step in one launch of one cluster,
+// for small grids (SMALL_CELLS): their lists hold few cells, and nine launches of
+// 2 to 3 us each were a third of the step.  Rounds are separated by the cluster's
+// barrier; every block reads the same counts after it, so all leave the loop in
+// the same round.
+constexpr int TAIL_BLOCKS = 8;
+__device__ __forceinline__ void cluster_barrier()
+{
+  __threadfence();
+  asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+  __threadfence();
+}
+template <bool G75>
+__global__ void __cluster_dims__(TAIL_BLOCKS, 1, 1) __launch_bounds__(LIST_THREADS) k_tail(StepArgs a)
+{
+  __shared__ long long q[2 * LIST_THREADS];
+  __shared__ int qn;
+  for (int r = 0; r < MAX_REPAIR; ++r) {
+    if (__ldcg(a.lcount + r) == 0) break;
+    repair_round<G75>(a, r, q, qn);
+    cluster_barrier();
+    update_round<SYS_EULER, false>(a, r);
+    cluster_barrier();
+  }
+  for (int d = blockIdx.x * blockDim.x + threadIdx.x; d < a.n_domains; d += gridDim.x * blockDim.x) finish_one(a, d);
+}
+
+// --------------------------------------------------------------- advection
+// One whole step of every domain in one launch: each cell forms the fluxes of
+// both its interfaces (the upwind cell's trace translated; twice the work of a
+// flux each, against three launches), and the first cell's thread keeps the
+// domain's books and forms its next time step, in the other buffer of ds (every
+// thread reads this step's).  Measured on 100 cells: 10 us a step in four
+// launches before.
+template <int M, bool NL>
+__global__ void __launch_bounds__(256) k_adv_step(StepArgs a, DomStep* next)
+{
+  const long long gi = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (gi >= a.ncell) return;
+  const int d = a.cell_dom[gi];
+  const DomStep r = a.ds[d];
+  const long long c0 = a.cell_off[d], i0 = a.if_off[d];
+  const int N = (int)(a.cell_off[d + 1] - c0), bc = a.bc[d], i = (int)(gi - c0);
+  const int jr = bc == 0 && i == N - 1 ? 0 : i + 1;
+  if (!r.active) {
+    a.avg_new[gi] = a.avg[gi];
+    a.ifc_new[i0 + i] = a.ifc[i0 + i];
+    if (bc != 0 && i == N - 1) a.ifc_new[i0 + N] = a.ifc[i0 + N];
+  } else {
+    const double lam = a.ph.lambda;
+    const bool pos = lam > 0.0;
+    double F[2], g[2];
+#pragma unroll 1
+    for (int e = 0; e < 2; ++e) {
+      // the upwind cell of the left (e = 0) or right (e = 1) interface, or the ghost
+      int c = i + e - (pos ? 1 : 0);
+      if (bc == 0) c = c < 0 ? N - 1 : (c == N ? 0 : c);
+      double em[1][M + 1], ep[1][M + 1];
+      bool fb;
+      if (c >= 0 && c < N) {
+        cell_edges<SYS_ADV, M, NL>(a, c0, i0, N, bc, c, em, ep, fb);
+      } else {
+        ghost_edge<SYS_ADV, M>(a, c0, c < 0 ? 0 : N - 1, em);
+#pragma unroll
+        for (int k = 0; k <= M; ++k) ep[0][k] = em[0][k];
+      }
+      double f, v;
+      grp_adv<M>(lam, r.nu, ep[0], em[0], f, v);
+      if (e == 0) { F[0] = f; g[0] = v; } else { F[1] = f; g[1] = v; }
+    }
+    a.avg_new[gi] = a.avg[gi] - r.nu * (F[1] - F[0]);
+    a.ifc_new[i0 + i] = g[0];
+    if (bc != 0 && i == N - 1) a.ifc_new[i0 + jr] = g[1];
+  }
+  if (i == 0) {
+    if (r.active) {
+      a.t[d] = r.last ? a.t_end : a.t[d] + r.dt;
+      a.nstep[d] += 1;
+      a.dt_prev[d] = r.dt_cfl;
+      a.stats[(long long)d * NSTATS + S_STEPS] += 1;
+    }
+    next[d] = domain_step(a, d);
+  }
 }
 
 // ------------------------------------------------------------------ batched
@@ -1610,10 +1775,30 @@ __global__ void __launch_bounds__(256) k_post(StepArgs a, const int* __restrict_
 
 // ------------------------------------------------------------------ init
 // Initial interface data: classical Riemann state of the one-sided limits.
+// Everything grp_set_initial clears, in one launch.
+static __global__ void k_reset(StepArgs a)
+{
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < a.nif) a.low[i] = 0;
+  if (i < a.ncell) a.troubled[i] = 0;
+  if (i < LCOUNT) a.lcount[i] = 0;
+  if (i < a.n_domains) {
+    a.t[i] = 0.0;
+    a.dt_prev[i] = 0.0;
+    a.nstep[i] = 0;
+    a.status[i] = 0;
+    a.smax_bits[i] = 0ull;
+    a.slow32[i] = 0u;
+    a.inad[i] = 0;
+    a.fail[i] = 0;
+    for (int p = 0; p <= MAX_REPAIR; ++p) a.bad[p * a.n_domains + i] = 0;
+    for (int k = 0; k < NSTATS; ++k) a.stats[i * NSTATS + k] = 0ull;
+  }
+}
+
 // The admissibility flags of given interface data.
 static __global__ void k_adm(double g, long long nif, const double* ifc, unsigned char* adm)
 {
-  chain_wait();
   const long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (j < nif) adm[j] = admissible(g, ifc[j], ifc[nif + j], ifc[2 * nif + j]) ? 1 : 0;
 }

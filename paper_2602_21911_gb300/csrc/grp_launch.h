@@ -7,29 +7,6 @@
 namespace grp {
 struct StepArgs;
 
-// Launches of a step's kernels; each begins with chain_wait.
-#ifdef __CUDACC__
-__device__ __forceinline__ void chain_wait()
-{
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-}
-template <typename... P, typename... A>
-inline cudaError_t chain(void (*kernel)(P...), unsigned grid, unsigned block, cudaStream_t s, A... args)
-{
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t c = {};
-  c.gridDim = dim3(grid);
-  c.blockDim = dim3(block);
-  c.stream = s;
-  c.attrs = at;
-  c.numAttrs = 0;
-  return cudaLaunchKernelEx(&c, kernel, P(args)...);
-}
-#endif
-
 // One launch of the persistent batched kernel.
 struct BatchLaunch {
   const StepArgs& a;
@@ -40,6 +17,10 @@ struct BatchLaunch {
 };
 
 cudaError_t launch_flux_adv(const StepArgs& a, cudaStream_t s);
+// one whole advection step; next: the time steps of the step after it
+struct DomStep;
+cudaError_t launch_adv_step(const StepArgs& a, DomStep* next, cudaStream_t s);
+cudaError_t launch_adv_step_nl(const StepArgs& a, DomStep* next, cudaStream_t s);
 cudaError_t launch_flux_adv_nl(const StepArgs& a, cudaStream_t s);
 cudaError_t launch_batch_adv_nl(const BatchLaunch& L, cudaStream_t s);
 cudaError_t launch_flux_euler_m1_nl(const StepArgs& a, cudaStream_t s);

@@ -53,7 +53,7 @@ struct Words {
   unsigned long long stats[NSTATS];
   int nstep, fail;
   int bad[MAX_REPAIR + 1], inad, any_bad[MAX_REPAIR + 1];
-  int lcount[2 * (MAX_REPAIR + 1)];
+  int lcount[LCOUNT];
   unsigned char bc;
 };
 constexpr size_t SCRATCH_BYTES = align256(OFF_WORDS + sizeof(Words));
@@ -74,7 +74,6 @@ unsigned char* g_scratch_addr[MAX_DEVICES];
 // Zeroes what must start at zero and writes the index tables and words.
 __global__ void k_noalloc_setup(unsigned char* base, int N, int nif, double dx, int bc, double t)
 {
-  chain_wait();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   int* cell_dom = (int*)(base + OFF_CELL_DOM);
   int* if_dom = (int*)(base + OFF_IF_DOM);
@@ -89,7 +88,7 @@ __global__ void k_noalloc_setup(unsigned char* base, int N, int nif, double dx, 
     for (int k = 0; k < NSTATS; ++k) w->stats[k] = 0ull;
     w->nstep = 0; w->out.status = 0; w->fail = 0;
     for (int p = 0; p <= MAX_REPAIR; ++p) { w->bad[p] = 0; w->any_bad[p] = 0; }
-    for (int p = 0; p < 2 * (MAX_REPAIR + 1); ++p) w->lcount[p] = 0;
+    for (int p = 0; p < LCOUNT; ++p) w->lcount[p] = 0;
     w->inad = 0;
     w->bc = (unsigned char)bc;
   }
@@ -147,8 +146,8 @@ extern "C" int grp_step_noalloc(int system, double lambda, double gamma, int M, 
   const double dx = (x_right - x_left) / N;
   Words* w = (Words*)(base + OFF_WORDS);
 
-  const unsigned tc = spread(N, 256), lb = list_blocks(N);
-  chain(k_noalloc_setup, nblk(nif, 256), 256, s, base, N, nif, dx, bc, t);
+  const unsigned tc = spread(N, 256), lb = LIST_BLOCKS;
+  k_noalloc_setup<<<nblk(nif, 256), 256, 0, s>>>(base, N, nif, dx, bc, t);
 
   StepArgs a;
   a.sys = system; a.M = M; a.C = system == GRP_EULER_IDEAL ? 3 : 1;
@@ -161,9 +160,7 @@ extern "C" int grp_step_noalloc(int system, double lambda, double gamma, int M, 
   a.dx = &w->dx; a.bc = &w->bc;
   a.avg = avg_in; a.avg_new = avg_out; a.ifc = iface_in; a.ifc_new = iface_out;
   a.flux = (double*)(base + OFF_FLUX);
-  a.pold = nullptr;
-  a.rp32 = (float2*)(base + OFF_POLD);
-  a.gm1f = (float)a.ph.gm1; a.gammaf = (float)a.ph.gamma; a.h_gm1f = (float)a.ph.h_gm1;
+  a.pold = (double*)(base + OFF_POLD);
   a.ds = (DomStep*)(base + OFF_DS);
   a.low = base + OFF_LOW; a.troubled = base + OFF_TROUBLED;
   a.t = &w->out.t; a.dt_prev = &w->dt_prev; a.nstep = &w->nstep; a.status = &w->out.status;
@@ -176,20 +173,25 @@ extern "C" int grp_step_noalloc(int system, double lambda, double gamma, int M, 
 
   // the flat step sequence of grp_step
   const bool euler = system == GRP_EULER_IDEAL;
-  if (euler) chain(k_speed, nblk(N, tc), tc, s, a);    // N <= SPEED_SMALL
-  chain(k_dt, 1, 32, s, a);
+  const bool small = euler && N <= SMALL_CELLS;
+  if (euler) k_speed<<<nblk(N, tc), tc, 0, s>>>(a, small ? 1 : 0);    // N <= SPEED_SMALL
+  if (!small) k_dt<<<1, 32, 0, s>>>(a);
   if (flux_dispatch(a, s) != cudaSuccess) return GRP_E_CUDA;
   if (euler) {
-    chain(k_update<SYS_EULER>, nblk(N, tc), tc, s, a, -1);
-    for (int r = 0; r < MAX_REPAIR; ++r) {
-      if (gamma == 1.4) chain(k_repair_list<true>, lb, LIST_THREADS, s, a, r);
-      else chain(k_repair_list<false>, lb, LIST_THREADS, s, a, r);
-      chain(k_update_list<SYS_EULER>, lb, LIST_THREADS, s, a, r);
+    k_update<SYS_EULER, false><<<nblk(N, tc), tc, 0, s>>>(a, -1);
+    if (small) {
+      if (gamma == 1.4) k_tail<true><<<TAIL_BLOCKS, LIST_THREADS, 0, s>>>(a);
+      else k_tail<false><<<TAIL_BLOCKS, LIST_THREADS, 0, s>>>(a);
+    }
+    for (int r = 0; r < MAX_REPAIR && !small; ++r) {
+      if (gamma == 1.4) k_repair_list<true><<<lb, LIST_THREADS, 0, s>>>(a, r);
+      else k_repair_list<false><<<lb, LIST_THREADS, 0, s>>>(a, r);
+      k_update_list<SYS_EULER, false><<<lb, LIST_THREADS, 0, s>>>(a, r);
     }
   } else {
-    chain(k_update<SYS_ADV>, nblk(N, tc), tc, s, a, -1);
+    k_update<SYS_ADV, false><<<nblk(N, tc), tc, 0, s>>>(a, -1);
   }
-  chain(k_finish, 1, 32, s, a);
+  if (!small) k_finish<<<1, 32, 0, s>>>(a);
   if (cudaGetLastError() != cudaSuccess) return GRP_E_CUDA;
   Result r;
   if (cudaMemcpyAsync(&r, &w->out, sizeof r, cudaMemcpyDeviceToHost, s) != cudaSuccess) return GRP_E_CUDA;

@@ -79,3 +79,13 @@ def test_riemann_problems_of_all_strengths(M, recon):
     for k, du in enumerate((0.01, 0.3, 1.0, -0.01, -0.3, -1.0)):
         prob, avg, lm, lp = I.riemann_problem(64, (1.0, -du, 1.0), (0.8 + 0.1 * k, du, 1.1), M=M, cfl=0.7)
         check_parity(dict(prob, recon=recon), avg, lm, lp, 25, DISC_TOL)
+
+
+@pytest.mark.parametrize("M,recon,N", [(2, 0, 9728), (2, 0, 9729), (2, 0, 19455), (2, 0, 19456), (4, 0, 19456),
+                                       (1, 0, 29183), (1, 0, 29184), (3, 0, 29184), (1, 1, 29184), (2, 1, 29184),
+                                       (3, 1, 29184)])
+def test_open_ends_around_the_sizes_where_the_pass_changes(M, recon, N):
+    """A strong jump (into the format's second pass, and repaired) and two open
+    ends, at both sides of every line of the dispatch for single domains."""
+    prob, avg, lm, lp = I.riemann_problem(N, (1.0, 0.4, 1.0), (0.2, -0.5, 0.1), M=M)
+    check_parity(dict(prob, recon=recon), avg, lm, lp, 6, DISC_TOL)
