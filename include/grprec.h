@@ -141,7 +141,8 @@ typedef struct {
  * 1.9], at degrees 1 and 3 and for GRPrecNL up to degree 3 with gamma = 7/5 and a
  * classical Newton start, where a Riemann problem counts 5 iterations in the
  * statistics; interfaces that leave that format's range are solved in FP64 by the
- * second kernel.
+ * second kernel.  The interface problems of the DET solver are solved in the
+ * format under the same conditions, at every degree and size.
  * Errors: GRP_E_INVALID_ARG for any field outside its range, GRP_E_CUDA.
  */
 int grp_create(grp_ctx **out, const grp_problem *p);

@@ -317,7 +317,11 @@ __global__ void __launch_bounds__(128) k_det_resume(StepArgs a, double* __restri
 // (Gauss quadrature over the M+1 time nodes) and the interface datum (the
 // state at the end of the step).  One thread per interface, full warps at the
 // statistics.
-template <int SYS, int M, bool G75>
+// FX: the problems in 64-bit fixed point (gamma = 7/5), FP64 for those that leave
+// its range: the kernel is bound by the FP64 pipe.  4,096 domains at degree 2: the
+// step 3.72 ms with all of it in FP64, 2.98 ms so (1,000 domains 1.79 and 1.58 ms,
+// at degree 1 0.83 and 0.66 ms); 20 domains 0.80 and 0.77 ms, so every size takes it.
+template <int SYS, int M, bool G75, bool FX>
 __global__ void __launch_bounds__(128) k_det_flux(StepArgs a, const double* __restrict__ ed)
 {
   constexpr int n = M + 1, C = SYS == SYS_EULER ? 3 : 1;
@@ -348,7 +352,12 @@ __global__ void __launch_bounds__(128) k_det_flux(StepArgs a, const double* __re
           QL[c] = cl < 0 ? a.avg[c * a.ncell + c0] : ed[det_idx(M, C, a.ncell, 1, g, c, c0 + cl)];
           QR[c] = cr < 0 ? a.avg[c * a.ncell + c0 + N - 1] : ed[det_idx(M, C, a.ncell, 0, g, c, c0 + cr)];
         }
-        if (SYS == SYS_ADV) {
+        bool newton = false, done = false;
+        if (FX) done = fixed::riemann_flux(a.fx, a.ph.gm1, QL, QR, Q0, F, newton);
+        if (FX && done) {
+          iters += newton ? (int)FIXED_ITERS : 0;
+          st[2] += 1;
+        } else if (SYS == SYS_ADV) {
           const double lam = a.ph.lambda;
           Q0[0] = lam > 0.0 ? QL[0] : (lam < 0.0 ? QR[0] : 0.5 * (QL[0] + QR[0]));
         } else {
@@ -362,7 +371,7 @@ __global__ void __launch_bounds__(128) k_det_flux(StepArgs a, const double* __re
           if (rs != ST_OK) { fo = true; break; }
         }
         if (g < n) {
-          phys_flux<SYS>(a.ph, Q0, F);
+          if (!FX || !done) phys_flux<SYS>(a.ph, Q0, F);
 #pragma unroll
           for (int c = 0; c < C; ++c) Fs[c] += T.w[g] * F[c];
         } else {
@@ -430,8 +439,10 @@ template <int SYS, int M>
 cudaError_t flux_launch(const StepArgs& a, const double* ed, cudaStream_t s)
 {
   const unsigned g = (unsigned)((a.nif + 127) / 128);
-  if (SYS == SYS_EULER && a.ph.gamma == 1.4) k_det_flux<SYS, M, true><<<g, 128, 0, s>>>(a, ed);
-  else k_det_flux<SYS, M, false><<<g, 128, 0, s>>>(a, ed);
+  constexpr bool E = SYS == SYS_EULER;
+  if (E && fixed_riemann(a)) k_det_flux<SYS, M, E, E><<<g, 128, 0, s>>>(a, ed);
+  else if (E && a.ph.gamma == 1.4) k_det_flux<SYS, M, E, false><<<g, 128, 0, s>>>(a, ed);
+  else k_det_flux<SYS, M, false, false><<<g, 128, 0, s>>>(a, ed);
   return cudaGetLastError();
 }
 

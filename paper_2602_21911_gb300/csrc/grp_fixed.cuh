@@ -799,5 +799,34 @@ GRP_HD __forceinline__ bool grp_traces(const Consts& K, double dgm1, double nu, 
   return evolve<M>(K, v, w, L, R, nu, dgm1 * to_double(w.Q[2], v.sE - 61), G, ok, F, gnew);
 }
 
+// Godunov state Q0 and its flux F of QL | QR in FP64 (gamma = 7/5).  false: outside
+// the format's range (inadmissible data among it), nothing to be used.
+GRP_HD __forceinline__ bool riemann_flux(const Consts& K, double dgm1, const double QL[3], const double QR[3],
+                                         double Q0[3], double F[3], bool& newton)
+{
+  bool ok = true;
+  Guard G;
+  const Units v = make_units(QL[0], QL[2], ok);
+  State w, a, b;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const Scale s = make_scale(61 - (c == 0 ? v.sr : c == 1 ? v.sm : v.sE));
+    a.Q[c] = G.chk<60>(to_fixed(QL[c], s, ok));
+    b.Q[c] = G.chk<60>(to_fixed(QR[c], s, ok));
+  }
+  newton = !(a.Q[0] == b.Q[0] && a.Q[1] == b.Q[1] && a.Q[2] == b.Q[2]);
+  riemann(K, a, b, w, G);
+  Q0[0] = to_double(w.Q[0], v.sr - 61);
+  Q0[1] = to_double(w.Q[1], v.sm - 61);
+  Q0[2] = to_double(w.Q[2], v.sE - 61);
+  const double u = to_double(w.u, v.ev - 61);
+  // (at rest the pressure must not depend on the interface's units)
+  const double ps = w.u == 0 ? dgm1 * Q0[2] : to_double(w.p, v.sE - 61);
+  F[0] = Q0[1];
+  F[1] = fma(Q0[1], u, ps);
+  F[2] = u * (Q0[2] + ps);
+  return ok && !G.out;
+}
+
 }  // namespace fixed
 }  // namespace grp

@@ -89,3 +89,15 @@ def test_open_ends_around_the_sizes_where_the_pass_changes(M, recon, N):
     ends, at both sides of every line of the dispatch for single domains."""
     prob, avg, lm, lp = I.riemann_problem(N, (1.0, 0.4, 1.0), (0.2, -0.5, 0.1), M=M)
     check_parity(dict(prob, recon=recon), avg, lm, lp, 6, DISC_TOL)
+
+
+@pytest.mark.parametrize("M", [1, 2, 3, 4])
+def test_predictor_solver_riemann_problems(M):
+    """The interface problems of the DET solver: weak and strong waves, flow in
+    both directions, and data that leave the format."""
+    for du, ratio in ((0.0, 0.9), (0.3, 1.1), (-0.5, 0.5), (1.0, 0.8), (-3.0, 0.01)):
+        prob, avg, lm, lp = I.riemann_problem(65, (1.0, -du, 1.0), (ratio, du, 1.1 * ratio), M=M, cfl=0.5)
+        check_parity(dict(prob, solver=1), avg, lm, lp, 8, DISC_TOL)
+    for u in (0.4, -2.5):
+        p, a, lo, hi = _wave(33, u, mass=3.0, speed=0.7, M=M)
+        check_parity(dict(p, solver=1), a, lo, hi, 8, SMOOTH_TOL)
