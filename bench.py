@@ -142,7 +142,8 @@ def source_digest():
 def profiled(cells, kname):
     """From the committed ncu summary of the dominant kernel (the flux phase):
     DRAM bytes per launch, scaled from its workload to this one by cell count,
-    and the executed FP64 flops (dadd + dmul + 2 dfma) per cell-update.  None
+    and the executed 64-bit operations (FP64 dadd + dmul + 2 dfma, and the
+    fixed-point products and sums) per cell-update.  None
     when the kernel source has changed since the capture or the summary is of
     another kernel."""
     if not os.path.exists(PROFILE):
@@ -749,9 +750,11 @@ def main():
                             "peak_source": "measured FP64 FMA-chain probe (grp_probe_fp64_peak), this GPU",
                             "basis": basis,
                             "flops_per_cell_update": ex_flops if prof else flops,
-                            "flops_note": "executed = the kernels' own FP64 flops per cell-update (dadd + dmul + "
-                                          "2 dfma, ncu, committed summary of the same source) over the live "
-                                          "CUDA-event duration of the flux phase; algorithmic = the CPU "
+                            "flops_note": "executed = the kernels' own 64-bit operations per cell-update (FP64 dadd + "
+                                          "dmul + 2 dfma, ncu, and the fixed-point products and sums of the first "
+                                          "pass, which run on the integer pipes: committed summary of the same "
+                                          "source) over the live CUDA-event duration of the flux phase, against the "
+                                          "FP64 peak (fixed point can exceed it); algorithmic = the CPU "
                                           "oracle's operation count, a costlier formulation of the same "
                                           "arithmetic (an upper bound)",
                             "algorithmic": {"flops_per_cell_update": flops, "achieved": alg / 1e12,
