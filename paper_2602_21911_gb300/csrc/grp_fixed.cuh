@@ -349,11 +349,15 @@ struct State {
   fx Q[3];                     // rho, m, 2 E
   fx iv, u, p, Ep, c, y;       // 1/(32 rho), velocity, 2 p, 2 (E + p), sound speed, 1/(8 c)
 };
-// ... the velocity and pressure of its conserved values
-GRP_HD __forceinline__ void primitive(const Consts& K, State& w)
+// ... the velocity and pressure of its conserved values.  In the state's own units
+// an admissible one has |u| < 1 (m^2 < 2 E rho); FOREIGN: in units that may be
+// another state's, and not known to be admissible, the product is tested before it
+// can wrap (|m| < 1/2 and rho >= 1/16 leave |u| up to 8).
+template <bool FOREIGN>
+GRP_HD __forceinline__ void primitive(const Consts& K, State& w, Guard& G)
 {
   w.iv = recip32(w.Q[0]);
-  w.u = mul_full<56>(w.Q[1], w.iv);                             // |u| < 1: m^2 < 2 E rho
+  w.u = FOREIGN ? mul_full<56>(w.Q[1], w.iv, G) : mul_full<56>(w.Q[1], w.iv);
   w.p = mul<61>(K.gm1, sub(w.Q[2], mul<61>(w.Q[1], w.u)));      // 2 p = (gamma - 1)(2 E - m u)
 }
 // ... the rest, from those
@@ -459,14 +463,13 @@ GRP_HD __forceinline__ fx pressure(const State& s, fx c2, fx i10c, fx d, Guard& 
 // conserved values; their other members are formed here.
 GRP_HD __forceinline__ void riemann(const Consts& K, State& L, State& R, State& w, Guard& G)
 {
-  primitive(K, L);
-  primitive(K, R);
+  primitive<true>(K, L, G);
+  primitive<true>(K, R, G);
   const bool equal = L.Q[0] == R.Q[0] && L.Q[1] == R.Q[1] && L.Q[2] == R.Q[2];
   fx c2[2];
 #pragma unroll
   for (int k = 0; k < 2; ++k) {
     State& s = k ? R : L;
-    G.see<61>(s.u);
     G.out = G.out || s.Q[0] < (1ll << 57) || s.Q[0] >= (1ll << 60);
     c2[k] = mul_full<56, 61>(mul<61>(K.hgam, s.p), s.iv, G);
     // slower sound than 1/8: general path, unless there is no wave
@@ -749,7 +752,7 @@ GRP_HD __forceinline__ bool grp_linear(const Consts& K, double dgm1, double nu, 
   newton = false;
   double still_p;
   if (EQ) {
-    primitive(K, w);
+    primitive<false>(K, w, G);
     still_p = dgm1 * g[1][2];
   } else {
     // admissible at the far edges (rho > 0, 2 E rho - m^2 > 0); at the near ones the Riemann problem sees to it

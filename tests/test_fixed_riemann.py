@@ -1,0 +1,34 @@
+"""Fixed-point Riemann problems on the host (gamma = 7/5): independent left and
+right states over decades, strong waves, rough data and inadmissible sides,
+against quad precision and beside the FP64 path."""
+import os
+import platform
+import subprocess
+
+import pytest
+
+from paper_2602_21911_gb300 import build as B
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+FLUX, FLUX_BAD, TRACES, ROUGH, TRACES_BAD = range(5)
+
+
+@pytest.fixture(scope="module")
+def lines(tmp_path_factory):
+    if platform.machine() != "x86_64":
+        pytest.skip("quad precision by libquadmath: x86")
+    exe = str(tmp_path_factory.mktemp("fixed") / "check")
+    r = subprocess.run([B._nvcc()] + B.ARCH + ["-O2", "-std=c++17", "-I" + B.CSRC,
+                                               os.path.join(HERE, "fixed_riemann_check.cu"), "-lquadmath", "-o", exe],
+                       capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    out = subprocess.run([exe, "20000"], capture_output=True, text=True)
+    assert out.returncode == 0
+    return [[float(x) for x in line.split()] for line in out.stdout.splitlines()]
+
+
+def test_inadmissible_traces_are_left_to_the_general_path(lines):
+    got = [x for x in lines if x[0] == TRACES_BAD]
+    assert len(got) == 4
+    for line in got:
+        assert line[-1] == 0, line
