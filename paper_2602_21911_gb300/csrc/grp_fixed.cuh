@@ -544,6 +544,7 @@ GRP_HD __forceinline__ void riemann(const Consts& K, State& L, State& R, State& 
   w.u = own ? k.u : us;
   w.p = own ? k.p : ps;
   G.see<60>(w.Q[2]);
+  G.see<61>(w.u);
   G.out = G.out || w.Q[0] < (1ll << 57) || w.Q[0] >= (1ll << 60);
   w.iv = recip32(w.Q[0]);
 }
@@ -828,7 +829,7 @@ GRP_HD __forceinline__ bool riemann_flux(const Consts& K, double dgm1, const dou
   F[0] = Q0[1];
   F[1] = fma(Q0[1], u, ps);
   F[2] = u * (Q0[2] + ps);
-  return ok && !G.out;
+  return ok && !G.bad();
 }
 
 }  // namespace fixed

@@ -32,3 +32,10 @@ def test_inadmissible_traces_are_left_to_the_general_path(lines):
     assert len(got) == 4
     for line in got:
         assert line[-1] == 0, line
+
+
+def test_inadmissible_sides_of_a_flux_are_refused(lines):
+    got = [x for x in lines if x[0] == FLUX_BAD]
+    assert len(got) == 4
+    for line in got:
+        assert line[-1] == 0, line
