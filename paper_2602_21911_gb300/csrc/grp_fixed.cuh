@@ -431,9 +431,13 @@ GRP_HD __forceinline__ void derivatives(const Consts& K, const State& s, const f
 // velocity is the unknown: with d the velocity by which the gas of a side is
 // pulled away from it, its pressure is p_K (1 - d / (5 c))^7 through a rarefaction
 // (d > 0), and p_K + rho |d| w, w = 0.6 |d| + sqrt(0.36 d^2 + c^2) the speed of
-// the shock into the side, otherwise: no roots but that one.  Newton's iteration
-// in FP32 leaves 2^-21; two steps with the pressures in the format and the slope
-// from FP32 leave less than its last bits.
+// the shock into the side, otherwise: no roots but that one.  Three steps of
+// Newton's iteration in FP32 leave about 2^-21; two steps follow with the pressures
+// in the format and the FP32 slopes of the last point, which are off by 2^-20 and by
+// a few times the first of these steps.  That one is held below 2^-16 and the second
+// below 2^-40, so what is left is below 2^-53, and 2^-57 once FP32 has converged.
+// (Slopes of the point before the last, and no bound of the second step, left up to
+// 4e-8 of the state.)
 // ---------------------------------------------------------------------------
 GRP_HD __forceinline__ float to_f32(fx x) { return (float)x * 0x1p-61f; }
 
@@ -492,6 +496,8 @@ GRP_HD __forceinline__ void riemann(const Consts& K, State& L, State& R, State& 
     const float pl = pressure32(l, x, kl), pr = pressure32(r, fdu - x, kr);
     x += (pl - pr) / (kl + kr);
   }
+  pressure32(l, x, kl);                                          // the slopes there
+  pressure32(r, fdu - x, kr);
   // the side's gas must stay away from vacuum (q > 1/2) and the iteration finite
   G.out = G.out || !(x * l.i5c < 0.5f && (fdu - x) * r.i5c < 0.5f && fabsf(x) < 0.5f && fabsf(fdu - x) < 0.5f);
   const float xs = fabsf(x) < 0.5f ? x : 0.0f;
@@ -506,7 +512,8 @@ GRP_HD __forceinline__ void riemann(const Consts& K, State& L, State& R, State& 
   const float s2 = to_f32(sub(pl, pr)) * inv;
   // the last step along the tangents; p* from both sides alike (a mirrored problem
   // gives the mirrored state)
-  const float t2 = fabsf(s2) < 0x1p-16f ? s2 : 0.0f;
+  G.out = G.out || !(fabsf(s2) < 0x1p-40f);
+  const float t2 = fabsf(s2) < 0x1p-40f ? s2 : 0.0f;
   const fx ps = add(add(pl >> 1, pr >> 1), (fx)(0.5f * (kr - kl) * t2 * 0x1p61f));
   d = add(d, (fx)(t2 * 0x1p61f));
   const fx us = add(L.u, d);

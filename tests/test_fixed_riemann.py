@@ -39,3 +39,19 @@ def test_inadmissible_sides_of_a_flux_are_refused(lines):
     assert len(got) == 4
     for line in got:
         assert line[-1] == 0, line
+
+
+def _errors_below_fp64(got):
+    for kind, degree, spread, share, rms, mx, rms64, mx64, wrong in got:
+        # rms below FP64's; a single result is rounded to a double of up to twice
+        # its unit (2^-52 of rho a^2 / (gamma (gamma - 1)))
+        assert rms <= rms64, (degree, spread, rms, rms64)
+        assert mx <= max(mx64, 2.0 ** -52 * 2.0 / (1.4 * 0.4)), (degree, spread, mx, mx64)
+        assert wrong == 0, (degree, spread, wrong)
+
+
+def test_errors_of_the_flux_are_below_the_fp64_path(lines):
+    """Strong waves among them: every problem that is taken has converged."""
+    got = [x for x in lines if x[0] == FLUX]
+    assert len(got) == 4 and got[0][3] > 0.9
+    _errors_below_fp64(got)
