@@ -365,8 +365,11 @@ GRP_HD __forceinline__ void acoustic(const Consts& K, State& w, Guard& G)
 {
   w.Ep = add(w.Q[2], w.p);
   G.out = G.out || w.p < (1ll << 20);
-  // c^2 = gamma p / rho, kept at 1/64 or more: below that the flow is supersonic
+  // c^2 = gamma p / rho, kept at 1/64 or more.  In the state's own units the flow is
+  // supersonic below that (|u| > 0.4), and takes a side whole; in another state's (the
+  // star state of an expansion in those of its left trace) it need not be, and is left
   const fx c2 = mul_full<56>(mul<61>(K.hgam, w.p), w.iv, G), lo = ONE >> 6;
+  G.out = G.out || (c2 < lo && w.u < (ONE >> 3) && w.u > -(ONE >> 3));
   const fx c2l = c2 < lo ? lo : c2;
   w.y = rsqrt8(c2l);
   w.c = mul<58>(c2l, w.y);

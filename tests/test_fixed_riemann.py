@@ -55,3 +55,12 @@ def test_errors_of_the_flux_are_below_the_fp64_path(lines):
     got = [x for x in lines if x[0] == FLUX]
     assert len(got) == 4 and got[0][3] > 0.9
     _errors_below_fp64(got)
+
+
+@pytest.mark.parametrize("kind", [TRACES, ROUGH])
+def test_errors_of_the_grp_are_below_the_fp64_path(lines, kind):
+    """Of traces with independent sides and slopes up to four times their size, and
+    of rough averages and interface data."""
+    got = [x for x in lines if x[0] == kind]
+    assert len(got) == (12 if kind == TRACES else 8) and got[0][3] > 0.4
+    _errors_below_fp64([x for x in got if x[3] > 0.0])
