@@ -340,11 +340,14 @@ static __global__ void __launch_bounds__(256) k_speed32(StepArgs a)
       const float ir = __fdividef(1.0f, rf), u = mf * ir, cap = a.gm1f * Ef;
       const float p = a.gm1f * fmaf(-0.5f * mf, u, Ef);
       const bool known = p > cap * 0x1p-9f;
-      const float au = fabsf(u), s = au + __fsqrt_rn(a.gammaf * (known ? p : cap * 0x1p-8f) * ir);
+      const float c2 = a.gammaf * (known ? p : cap * 0x1p-8f) * ir;
+      const float au = fabsf(u), s = au + __fsqrt_rn(c2);
       const float tol = p > cap * 0x1p-4f ? 0x1p-15f : 0x1p-10f;
       float sl = (known ? s : au) * (1.0f - tol), su = s * (1.0f + tol);
-      if (!(rf > 1e-30f && cap > 1e-30f && su < 1e30f)) { sl = 0.0f; su = INFINITY; }
-      a.rp32[gi] = make_float2(rf, known && su < 1e30f ? p : NAN);
+      // (the fast reciprocal is 0 from 2^126 on; c^2 must not have vanished either)
+      const bool held = rf > 1e-30f && rf < 1e30f && cap > 1e-30f && c2 > 1e-30f && su < 1e30f;
+      if (!held) { sl = 0.0f; su = INFINITY; }
+      a.rp32[gi] = make_float2(rf, known && held ? p : NAN);
       a.sup32[gi] = su;
       low = __float_as_uint(sl);
     }
