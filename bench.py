@@ -139,11 +139,16 @@ def source_digest():
     return h.hexdigest()[:16]
 
 
+# Measured rates of the fixed-point operations per SM and cycle, each alone: a 64-bit
+# product from three 32-bit ones, a 64-bit sum.
+FIXED_PRODUCTS_PER_CYCLE, FIXED_SUMS_PER_CYCLE = 7.5, 42.0
+
+
 def profiled(cells, kname):
     """From the committed ncu summary of the dominant kernel (the flux phase):
     DRAM bytes per launch, scaled from its workload to this one by cell count,
-    and the executed 64-bit operations (FP64 dadd + dmul + 2 dfma, and the
-    fixed-point products and sums) per cell-update.  None
+    and per cell-update the executed 64-bit operations (all of them, and apart:
+    FP64 dadd + dmul + 2 dfma; fixed-point products and sums).  None
     when the kernel source has changed since the capture or the summary is of
     another kernel."""
     if not os.path.exists(PROFILE):
@@ -155,8 +160,21 @@ def profiled(cells, kname):
             kv[k.strip()] = v.strip()
     if kv.get("source_digest") != source_digest() or kv.get("bench_kernel") != kname:
         return None
+    per_cell = float(kv["interfaces_per_launch"]) / float(kv["cells_per_launch"])
+    fp64, products, sums = (per_cell * float(kv[k]) for k in ("fp64_flops_per_interface",
+                                                             "fixed_point_products_per_interface",
+                                                             "fixed_point_sums_per_interface"))
     return {"traffic": float(kv["dram_bytes_per_launch"]) * cells / float(kv["cells_per_launch"]),
-            "executed_flops_per_cell_update": float(kv["executed_fp64_flops_per_cell_update"])}
+            "executed_flops_per_cell_update": fp64 + 2.0 * products + sums,
+            "fp64_flops": fp64, "products": products, "sums": sums,
+            "pass1_alu_pipe_busy_pct": float(kv["pass1_alu_pipe_busy_pct"].split()[0])}
+
+
+def fixed_point_peak(products, sums, sms, sm_mhz):
+    """Fixed-point operations (products and sums) per second of the whole GPU at
+    their measured rates, in this mix."""
+    cycles = products / FIXED_PRODUCTS_PER_CYCLE + sums / FIXED_SUMS_PER_CYCLE
+    return (products + sums) / cycles * sms * sm_mhz * 1e6
 
 
 def workload(args, rank, world):
@@ -738,27 +756,33 @@ def main():
         dur = flux_ms / flux_n * 1e-3                 # one flux phase (both passes), CUDA events
         alg = flops * per_launch_updates / dur
         prof = profiled(int(prob["n_cells"].sum()), kname)
+        algorithmic = {"flops_per_cell_update": flops, "achieved": alg / 1e12, "unit": "TFLOP/s",
+                       "note": "the CPU oracle's operation count, a costlier formulation of the same arithmetic"}
+        fp64_source = "measured FP64 FMA-chain probe (grp_probe_fp64_peak), this GPU"
         if prof:
-            ex_flops = prof["executed_flops_per_cell_update"]
-            ach, basis = ex_flops * per_launch_updates / dur, "executed"
+            sms = torch.cuda.get_device_properties(local).multi_processor_count
+            mhz = line["clocks"]["sm_mhz"] or 2070.0
+            fx_peak = fixed_point_peak(prof["products"], prof["sums"], sms, mhz)
+            fx = (prof["products"] + prof["sums"]) * per_launch_updates / dur
+            f64 = prof["fp64_flops"] * per_launch_updates / dur
+            line["roofline"] = {"bound": "alu", "achieved": fx / 1e12, "peak": fx_peak / 1e12,
+                                "unit": "T fixed-point operations/s", "frac": fx / fx_peak,
+                                "traffic": prof["traffic"], "kernel": kname, "basis": "executed",
+                                "peak_source": "measured rates per SM and cycle: %g 64-bit products, %g sums; %d SMs "
+                                               "at %g MHz" % (FIXED_PRODUCTS_PER_CYCLE, FIXED_SUMS_PER_CYCLE, sms, mhz),
+                                "per_cell_update": {"products": prof["products"], "sums": prof["sums"],
+                                                    "fp64_flops": prof["fp64_flops"]},
+                                "note": "products and sums of the fixed-point first pass (counted from a run of its "
+                                        "code) over the live CUDA-event duration of the whole flux phase, both passes; "
+                                        "the second pass is FP64 and bound by latency",
+                                "pass1_alu_pipe_busy_pct": prof["pass1_alu_pipe_busy_pct"],
+                                "fp64": {"achieved": f64 / 1e12, "peak": peak / 1e12, "unit": "TFLOP/s",
+                                         "frac": f64 / peak, "peak_source": fp64_source},
+                                "algorithmic": algorithmic}
         else:
-            ex_flops, ach, basis = None, alg, "algorithmic"
-        line["roofline"] = {"bound": "alu", "achieved": ach / 1e12, "peak": peak / 1e12, "unit": "TFLOP/s",
-                            "frac": ach / peak,
-                            "traffic": prof["traffic"] if prof else None,
-                            "kernel": kname,
-                            "peak_source": "measured FP64 FMA-chain probe (grp_probe_fp64_peak), this GPU",
-                            "basis": basis,
-                            "flops_per_cell_update": ex_flops if prof else flops,
-                            "flops_note": "executed = the kernels' own 64-bit operations per cell-update (FP64 dadd + "
-                                          "dmul + 2 dfma, ncu, and the fixed-point products and sums of the first "
-                                          "pass, which run on the integer pipes: committed summary of the same "
-                                          "source) over the live CUDA-event duration of the flux phase, against the "
-                                          "FP64 peak (fixed point can exceed it); algorithmic = the CPU "
-                                          "oracle's operation count, a costlier formulation of the same "
-                                          "arithmetic (an upper bound)",
-                            "algorithmic": {"flops_per_cell_update": flops, "achieved": alg / 1e12,
-                                            "frac": alg / peak}}
+            line["roofline"] = {"bound": "alu", "achieved": alg / 1e12, "peak": peak / 1e12, "unit": "TFLOP/s",
+                                "frac": alg / peak, "traffic": None, "kernel": kname, "peak_source": fp64_source,
+                                "basis": "algorithmic", "algorithmic": algorithmic}
     if not args.no_l1 and args.plain_domains > 0:
         line["l1"] = l1_measurements(args, local, stream, w, box)
     if not args.no_other:
