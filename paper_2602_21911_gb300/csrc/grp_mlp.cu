@@ -68,7 +68,12 @@ __global__ void __launch_bounds__(256) k_mlp_tiles(const float* __restrict__ w, 
   for (long long tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
     const long long base = tile * TILE;
     __syncthreads();                                // the weights are there; the last tile is done with
-    if (tid < TILE * MLP_NIN) S.X[tid] = base * MLP_NIN + tid < n * MLP_NIN ? x[base * MLP_NIN + tid] : 0.0f;
+    // (places past the end repeat the last sample with no weight: zeros would meet
+    // an infinite weight as 0 x infinity)
+    if (tid < TILE * MLP_NIN) {
+      const long long s = base + tid / MLP_NIN;
+      S.X[tid] = x[(s < n ? s : n - 1) * MLP_NIN + tid % MLP_NIN];
+    }
     __syncthreads();
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
