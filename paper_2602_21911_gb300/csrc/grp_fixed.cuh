@@ -1,5 +1,7 @@
-// The GRP at an interface with equal data (degrees 2 and 4 of the linear
-// reconstruction) in 64-bit fixed point, on the integer pipes.
+// The GRP at an interface in 64-bit fixed point, on the integer pipes: with equal
+// data (degrees 2 and 4 of the linear reconstruction), and for gamma = 7/5 with a
+// leading Riemann problem (degrees 1 and 3, GRPrecNL up to degree 3, and the
+// interface problems of the DET solver, which are that problem alone).
 //
 // Why: an SM of this GPU retires 2 FP64 lane-operations per cycle and 64
 // 32 x 32 -> 64 multiply-adds; one 64-bit fixed-point product costs three of
@@ -10,18 +12,20 @@
 // Precision.  Every interface has its own powers of two for length, time and
 // mass (exact scalings), so that its state sits at the top of the format: a
 // number x of the scaled problem is the integer x 2^61.  With V^2 a power of
-// four and x = E/(rho V^2) in [1/8, 1/2):
+// four and x = E/(rho V^2) in [1/8, 1/2) for the state that sets the units (the
+// interface datum of equal data, otherwise the left cell's average or trace):
 //   density  rho 2^-(er+2)          in [1/8, 1/4)   2^58..2^59 units
 //   momentum rho V as unit of rho   |m| < rho
 //   energy   2 E (twice the unit)   in [rho/4, rho) at least 2^56 units
 //   velocity u / V                  |u| < 1
-// A double of the interface's state converts exactly (its last bit is worth 8
-// units or more), a product is off by at most 2 units (its low x low partial
-// product is left out), so an operation's error is 2^-56 or less of the state
-// where an FP64 operation's is 2^-53.  Nothing wraps unseen: every operand of a
-// product is tested against its bound, and an interface that leaves the range
-// (a jump of more than about 4 between neighbours, sonic fields, a state near
-// vacuum) is solved in FP64 by the second pass instead.
+// A double of that state converts exactly (its last bit is worth 8 units or
+// more), a product is off by at most 2 units (its low x low partial product is
+// left out), so an operation's error is 2^-56 or less of the state where an FP64
+// operation's is 2^-53.  Every operand of a product is tested against its bound,
+// or bounded by tests before it, and an interface that leaves the range (a jump of
+// more than about 4 between neighbours, sonic fields, sound slower than V/8, an
+// iteration that has not converged, a state near vacuum or inadmissible) is solved
+// in FP64 instead: by the second pass, or in place (DET).
 #pragma once
 #include "grp_device.cuh"
 
@@ -513,8 +517,10 @@ GRP_HD __forceinline__ void riemann(const Consts& K, State& L, State& R, State& 
   d = add(d, (fx)(fabsf(s1) < 0x1p-16f ? s1 * 0x1p61f : 0.0f));
   const fx pl = pressure(L, c2[0], iL, d, G), pr = pressure(R, c2[1], iR, sub(du, d), G);
   const float s2 = to_f32(sub(pl, pr)) * inv;
-  // the last step along the tangents; p* from both sides alike (a mirrored problem
-  // gives the mirrored state)
+  // the last step along the tangents; p* from both sides alike, so that a mirrored
+  // problem in the same units gives the mirrored state.  (The units are the left
+  // side's: the mirror image of an interface agrees to the format's rounding, and
+  // near the bounds one of the two may be left to FP64 alone.)
   G.out = G.out || !(fabsf(s2) < 0x1p-40f);
   const float t2 = fabsf(s2) < 0x1p-40f ? s2 : 0.0f;
   const fx ps = add(add(pl >> 1, pr >> 1), (fx)(0.5f * (kr - kl) * t2 * 0x1p61f));
