@@ -318,9 +318,14 @@ __global__ void __launch_bounds__(128) k_det_resume(StepArgs a, double* __restri
 // state at the end of the step).  One thread per interface, full warps at the
 // statistics.
 // FX: the problems in 64-bit fixed point (gamma = 7/5), FP64 for those that leave
-// its range: the kernel is bound by the FP64 pipe.  4,096 domains at degree 2: the
-// step 3.72 ms with all of it in FP64, 2.98 ms so (1,000 domains 1.79 and 1.58 ms,
-// at degree 1 0.83 and 0.66 ms); 20 domains 0.80 and 0.77 ms, so every size takes it.
+// its range: the kernel is bound by the FP64 pipe.  An interface that has left the
+// range at one time node takes FP64 at the nodes after it (neighbouring nodes are
+// alike, and a warp pays for both where its lanes disagree).  Batches, half of the
+// domains with strong data, us per step all in FP64 / so: degree 2, 4,096 domains
+// 3,700 / 3,017, 1,000 domains 1,788 / 1,591, 400 domains 1,364 / 1,329, 20 domains
+// 847 / 856 (with every node tried anew 3,062, 1,623, 1,360 and 874); degree 1, 1,000
+// domains 799 / 671, 100 domains 386 / 401.  Smooth data gain at every size (wave of
+// 8,192 cells 128 / 101), as does one Sod tube (539 / 481), so every size takes it.
 template <int SYS, int M, bool G75, bool FX>
 __global__ void __launch_bounds__(128) k_det_flux(StepArgs a, const double* __restrict__ ed)
 {
@@ -343,7 +348,7 @@ __global__ void __launch_bounds__(128) k_det_flux(StepArgs a, const double* __re
       a.low[gj] = 0;
       const DetTab& T = c_det[M - 1];
       double Fs[3] = {0.0, 0.0, 0.0}, gnew[3] = {0.0, 0.0, 0.0};
-      bool fo = false;
+      bool fo = false, held = true;
       int iters = 0;
       for (int g = 0; g <= n && !fo; ++g) {
         double QL[3] = {0.0, 0.0, 0.0}, QR[3] = {0.0, 0.0, 0.0}, Q0[3], F[3];
@@ -353,7 +358,7 @@ __global__ void __launch_bounds__(128) k_det_flux(StepArgs a, const double* __re
           QR[c] = cr < 0 ? a.avg[c * a.ncell + c0 + N - 1] : ed[det_idx(M, C, a.ncell, 0, g, c, c0 + cr)];
         }
         bool newton = false, done = false;
-        if (FX) done = fixed::riemann_flux(a.fx, a.ph.gm1, QL, QR, Q0, F, newton);
+        if (FX && held) held = done = fixed::riemann_flux(a.fx, a.ph.gm1, QL, QR, Q0, F, newton);
         if (FX && done) {
           iters += newton ? (int)FIXED_ITERS : 0;
           st[2] += 1;
